@@ -21,8 +21,9 @@
  *   slow_v  float32 [N]     SlowMo velocity v
  *   grads   float32 or bfloat16 [W][N], read only, row i = worker i
  * Row stride is exactly N elements. All pointers must be 16-byte aligned.
- * The fast vectorised kernels run when N is a multiple of 4; any other N runs
- * a scalar path with the same results.
+ * The 128-bit kernels run when N is a multiple of 4; for any other N the rows
+ * start off a vector boundary and the reconcile loads pairs of columns (N even)
+ * or single ones (N odd), with the same results.
  *
  * Optimizer step (the paper's implementation: PyTorch SGD, momentum 0.9,
  * weight decay 5e-4; Sec. 4.2, Table 3), per element:

@@ -14,9 +14,9 @@ PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
 INCLUDE = ROOT / "include"
 CSRC = PKG / "csrc"
-SOURCES = [CSRC / "cpdp.cu"]
+SOURCES = [CSRC / "cpdp.cu", CSRC / "cpdp_ragged.cu"]
 DEPENDS = SOURCES + [CSRC / "cpdp_kernels.cuh", CSRC / "cpdp_shapes.cuh", CSRC / "cpdp_tma.cuh",
-                     CSRC / "cpdp_floor.cuh", CSRC / "cpdp_shuffle.cuh", INCLUDE / "cpdp.h"]
+                     CSRC / "cpdp_floor.cuh", CSRC / "cpdp_shuffle.cuh", CSRC / "cpdp_launch.cuh", INCLUDE / "cpdp.h"]
 LIBRARY = PKG / "libcpdp.so"
 CHECKED_LIBRARY = PKG / "libcpdp_checked.so"  # debug build: kernels count out-of-range indices
 BUILD_DIR = ROOT / "_build"
@@ -35,7 +35,7 @@ def nvcc_path() -> str:
 
 def nvcc_command(output: Path, sources=SOURCES, extra: list[str] | None = None) -> list[str]:
     return [nvcc_path(), "-O3", "-std=c++17", *ARCH, "-lineinfo",
-            "-Xcompiler", "-fPIC,-O2", "-shared", "-Xptxas", "-v",
+            "-Xcompiler", "-fPIC,-O2", "-shared", "-Xptxas", "-v", "--threads", "0",
             f"-I{INCLUDE}", f"-I{CSRC}", "-o", str(output), *map(str, sources), *(extra or [])]
 
 

@@ -6,6 +6,7 @@
 #include "cpdp.h"
 #include "cpdp_floor.cuh"
 #include "cpdp_kernels.cuh"
+#include "cpdp_launch.cuh"
 #include "cpdp_shapes.cuh"
 #include "cpdp_shuffle.cuh"
 #include "cpdp_tma.cuh"
@@ -175,29 +176,9 @@ cpdp_status check_launch(cpdp_ctx* ctx, cudaError_t launched, const char* what) 
     return CPDP_OK;
 }
 
-// Launch `kernel` with kThreads threads per block on `s`. With the context's
-// programmatic dependent launch on, the launch may begin while the previous
-// grid on the stream drains; every kernel waits for that grid's completion
-// itself before touching memory (cpdp::pdl_wait_then_release).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_shaped(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                          cudaStream_t s, Args... args) {
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <typename... KArgs, typename... Args>
 cudaError_t launch(const cpdp_ctx* c, void (*kernel)(KArgs...), unsigned grid, cudaStream_t s, Args... args) {
-    return launch_shaped(c->pdl, kernel, grid, cpdp::kThreads, 0, s, args...);
+    return cpdp::launch_shaped(c->pdl, kernel, grid, cpdp::kThreads, 0, s, args...);
 }
 
 // Whether `s` is being captured into a CUDA graph (a query that is legal
@@ -337,8 +318,8 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
         return launch_vec4<cpdp::ReconcileShape<OPT, G, SS>, METHOD, OPT, SS, G>(c, g, sq, s, a, nq);
     }
     c->reconcile_kernel = "reconcile_scalar_kernel";
-    return launch(c, cpdp::reconcile_scalar_kernel<METHOD, OPT, SS, G>, cpdp::grid_for(c->N, cpdp::kThreads), s, c->params,
-                  c->mom, sq, g, c->anchor, c->slow_v, c->W, c->N, a);
+    return cpdp::launch_reconcile_ragged({c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
+                                          c->anchor, c->slow_v, a, s});
 }
 
 template <int METHOD, int OPT, typename G>
@@ -372,7 +353,7 @@ cudaError_t launch_reconcile_tma(cpdp_ctx* c, const float* grads, cudaStream_t s
     const int64_t withheld = c->tma_withheld_tile;
     c->tma_withheld_tile = -1;
     c->reconcile_kernel = "reconcile_tma_kernel";
-    return launch_shaped(c->pdl, cpdp::reconcile_tma_kernel, grid, cpdp::kTmaThreads, c->tma_smem, s, c->params,
+    return cpdp::launch_shaped(c->pdl, cpdp::reconcile_tma_kernel, grid, cpdp::kTmaThreads, c->tma_smem, s, c->params,
                          c->mom, grads, c->anchor, c->slow_v, c->W, c->N, c->tma_stages, withheld, a);
 }
 
@@ -389,7 +370,7 @@ cudaError_t launch_reconcile_shuffle(cpdp_ctx* c, const float* grads, cudaStream
 template <typename G, int CH, int MB>
 cudaError_t launch_floor_columns(float* params, float* mom, float* sq, const void* grads, float* anchor, float* slow_v,
                                  int W, int64_t nq, cudaStream_t s) {
-    return launch_shaped(true, cpdp::floor_columns_kernel<G, CH, MB>, cpdp::grid_for(nq, cpdp::kThreads),
+    return cpdp::launch_shaped(true, cpdp::floor_columns_kernel<G, CH, MB>, cpdp::grid_for(nq, cpdp::kThreads),
                          cpdp::kThreads, 0, s, params, mom, sq, static_cast<const G*>(grads), anchor, slow_v, W, nq);
 }
 
@@ -977,8 +958,10 @@ cpdp_status cpdp_bad_index_count(cpdp_ctx* ctx, int64_t* count) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpyFromSymbol(&seen, cpdp::bad_index_count, sizeof seen);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(cpdp::bad_index_count, &zero, sizeof zero);
+    unsigned long long ragged = 0;  // the other translation unit's own counter
+    if (e == cudaSuccess) e = cpdp::take_bad_indices_ragged(&ragged);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "reading the bad-index count");
-    *count = static_cast<int64_t>(seen);
+    *count = static_cast<int64_t>(seen + ragged);
 #else
     *count = -1;  // a release build checks no index
 #endif
@@ -1015,7 +998,7 @@ cpdp_status cpdp_floor_stream(const float* const* in, int n_in, const uint16_t* 
     }
     const int64_t nq = n >> 2;
     const unsigned g = grid != 0 ? grid : cpdp::grid_for(nq, cpdp::kThreads);
-    const cudaError_t e = launch_shaped(true, cpdp::floor_stream_kernel, g, cpdp::kThreads, 0,
+    const cudaError_t e = cpdp::launch_shaped(true, cpdp::floor_stream_kernel, g, cpdp::kThreads, 0,
                                         static_cast<cudaStream_t>(stream), rows, nq);
     const cudaError_t e2 = e != cudaSuccess ? e : cudaGetLastError();
     if (e2 != cudaSuccess) return set_error(nullptr, CPDP_ECUDA, "floor_stream launch: %s", cudaGetErrorString(e2));
@@ -1023,7 +1006,7 @@ cpdp_status cpdp_floor_stream(const float* const* in, int n_in, const uint16_t* 
 }
 
 cpdp_status cpdp_floor_empty(unsigned grid, void* stream) {
-    const cudaError_t e = launch_shaped(true, cpdp::floor_empty_kernel, grid != 0 ? grid : 1u, cpdp::kThreads, 0,
+    const cudaError_t e = cpdp::launch_shaped(true, cpdp::floor_empty_kernel, grid != 0 ? grid : 1u, cpdp::kThreads, 0,
                                         static_cast<cudaStream_t>(stream));
     const cudaError_t e2 = e != cudaSuccess ? e : cudaGetLastError();
     if (e2 != cudaSuccess) return set_error(nullptr, CPDP_ECUDA, "floor_empty launch: %s", cudaGetErrorString(e2));

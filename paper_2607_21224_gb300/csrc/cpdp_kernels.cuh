@@ -103,6 +103,11 @@ struct GradLoad<float> {
     using Words = float4;
     static __device__ __forceinline__ Words words(const float* g, int64_t q) { return vec4(g, q); }
     static __device__ __forceinline__ float4 widen(const Words& w) { return w; }
+    // a pair of elements (e2 indexes pairs) as two words, and a single element as one
+    static __device__ __forceinline__ void pair(const float* g, int64_t e2, float& a, float& b) {
+        const float2 u = __ldg(reinterpret_cast<const float2*>(g) + e2);
+        a = u.x, b = u.y;
+    }
 };
 
 template <>
@@ -123,6 +128,108 @@ struct GradLoad<bf16_bits> {
     static __device__ __forceinline__ float4 widen(const Words& u) {
         return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
                            __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+    }
+    static __device__ __forceinline__ uint32_t pair(const bf16_bits* g, int64_t e2) {
+        return __ldg(reinterpret_cast<const unsigned int*>(g) + e2);
+    }
+    static __device__ __forceinline__ uint32_t bits(const bf16_bits* g, int64_t e) {
+        return __ldg(reinterpret_cast<const unsigned short*>(g) + e);
+    }
+};
+
+// Which columns of a [W][N] array a thread owns, and how it reaches them in
+// one row. V is the widest load that every row's start allows: rows begin
+// every N elements, so 4 elements (16 bytes of float32) when N is a multiple
+// of 4, a pair when it is even, else a single one. n counts a row in units of
+// V elements; a thread owns the U units first, first + 32, ... (U * V <= 4), so
+// that the lanes of a warp read neighbouring units. Its columns sit in the
+// low U * V components of a float4; the others are 0 and take no part. Units
+// at or past n load as 0 and are not stored; with FULL there are none (with
+// one unit the caller's loop keeps it below n).
+template <int V, int U, typename Idx, bool FULL = U == 1>
+struct Columns {
+    static_assert((V == 4 || V == 2 || V == 1) && U >= 1 && U * V <= 4, "units of 4, 2 or 1 elements, 4 in all");
+    Idx n, first;
+    int W;
+
+    // index of unit k of row `row`, checked against `rows` rows
+    __device__ __forceinline__ Idx at(Idx row, int k, int rows) const {
+        return CPDP_IDX(row * n + first + (Idx)(32 * k), (Idx)rows * n);
+    }
+    __device__ __forceinline__ bool has(int k) const { return k < U && (FULL || first + (Idx)(32 * k) < n); }
+
+    __device__ __forceinline__ float4 load(const float* p, Idx row, int rows) const {
+        if constexpr (V == 4) {
+            return reinterpret_cast<const float4*>(p)[at(row, 0, rows)];
+        } else if constexpr (V == 2) {
+            const float2* p2 = reinterpret_cast<const float2*>(p);
+            float2 a = make_float2(0.f, 0.f), b = a;
+            if (has(0)) a = p2[at(row, 0, rows)];
+            if (has(1)) b = p2[at(row, 1, rows)];
+            return make_float4(a.x, a.y, b.x, b.y);
+        } else {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (has(0)) x.x = p[at(row, 0, rows)];
+            if (has(1)) x.y = p[at(row, 1, rows)];
+            if (has(2)) x.z = p[at(row, 2, rows)];
+            if (has(3)) x.w = p[at(row, 3, rows)];
+            return x;
+        }
+    }
+    __device__ __forceinline__ void store(float* p, Idx row, int rows, const float4& x) const {
+        if constexpr (V == 4) {
+            reinterpret_cast<float4*>(p)[at(row, 0, rows)] = x;
+        } else if constexpr (V == 2) {
+            float2* p2 = reinterpret_cast<float2*>(p);
+            if (has(0)) p2[at(row, 0, rows)] = make_float2(x.x, x.y);
+            if (has(1)) p2[at(row, 1, rows)] = make_float2(x.z, x.w);
+        } else {
+            if (has(0)) p[at(row, 0, rows)] = x.x;
+            if (has(1)) p[at(row, 1, rows)] = x.y;
+            if (has(2)) p[at(row, 2, rows)] = x.z;
+            if (has(3)) p[at(row, 3, rows)] = x.w;
+        }
+    }
+    __device__ __forceinline__ float4 load(const float* p, Idx row) const { return load(p, row, W); }
+    __device__ __forceinline__ void store(float* p, Idx row, const float4& x) const { store(p, row, W, x); }
+
+    // the gradient words of a row (GradLoad<G>::Words; widened when summed)
+    __device__ __forceinline__ float4 words(const float* g, Idx row) const {
+        if constexpr (V == 4) {
+            return GradLoad<float>::words(g, at(row, 0, W));
+        } else if constexpr (V == 2) {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (has(0)) GradLoad<float>::pair(g, at(row, 0, W), x.x, x.y);
+            if (has(1)) GradLoad<float>::pair(g, at(row, 1, W), x.z, x.w);
+            return x;
+        } else {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (has(0)) x.x = GradLoad<float>::one(g, at(row, 0, W));
+            if (has(1)) x.y = GradLoad<float>::one(g, at(row, 1, W));
+            if (has(2)) x.z = GradLoad<float>::one(g, at(row, 2, W));
+            if (has(3)) x.w = GradLoad<float>::one(g, at(row, 3, W));
+            return x;
+        }
+    }
+    __device__ __forceinline__ uint2 words(const bf16_bits* g, Idx row) const {
+        if constexpr (V == 4) {
+            return GradLoad<bf16_bits>::words(g, at(row, 0, W));
+        } else if constexpr (V == 2) {
+            uint2 u = make_uint2(0u, 0u);
+            if (has(0)) u.x = GradLoad<bf16_bits>::pair(g, at(row, 0, W));
+            if (has(1)) u.y = GradLoad<bf16_bits>::pair(g, at(row, 1, W));
+            return u;
+        } else {
+            uint32_t b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (has(k)) b[k] = GradLoad<bf16_bits>::bits(g, at(row, k, W));
+            return make_uint2(b[0] | (b[1] << 16), b[2] | (b[3] << 16));
+        }
+    }
+    template <typename G>
+    __device__ __forceinline__ float4 grads(const G* g, Idx row) const {
+        return GradLoad<G>::widen(words(g, row));
     }
 };
 
@@ -197,7 +304,7 @@ __device__ __forceinline__ void pdl_wait_then_release() {
 // theta_ref = theta0, v = 0, buf_i = 0 (and the AdamW second moments, when
 // `sq` is not null).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads)
+static __global__ void __launch_bounds__(kThreads)
 init_vec4_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
                  float* __restrict__ anchor, float* __restrict__ slow_v, const float* __restrict__ theta0,
                  int W, int64_t nq) {
@@ -219,7 +326,7 @@ init_vec4_kernel(float* __restrict__ params, float* __restrict__ mom, float* __r
     }
 }
 
-__global__ void __launch_bounds__(kThreads)
+static __global__ void __launch_bounds__(kThreads)
 init_scalar_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
                    float* __restrict__ anchor, float* __restrict__ slow_v, const float* __restrict__ theta0,
                    int W, int64_t N) {
@@ -350,148 +457,162 @@ constexpr int kMethodLocalSGD = 1;
 constexpr int kMethodDDP = 2;
 
 // Steps 2-3 of the reconcile below for the chunk of rows i0 .. i0 + CH - 1 of
-// column group c, the rows already in registers: each worker's optimizer step
-// (with gbar, or with its own gradient gw for LocalSGD), its state written
+// the thread's columns, the rows already in registers: each worker's optimizer
+// step (with gbar, or with its own gradient gw for LocalSGD), its state written
 // back or added to the state sums, its parameters written back (DDP) or added
 // to the parameter sum.
-template <int METHOD, int OPT, bool STATE_SYNC, int CH, typename Idx>
-__device__ __forceinline__ void reconcile_chunk(int i0, int W, Idx nq, Idx c, float4* p4, float4* m4, float4* s4,
-                                                const float4& gbar, const StepArgs& step, float4 (&th)[CH],
-                                                float4 (&bu)[CH], float4 (&sv)[CH], const float4 (&gw)[CH],
-                                                float4& tsum, float4& bsum, float4& ssum) {
+template <int METHOD, int OPT, bool STATE_SYNC, int CH, int V, int U, typename Idx, bool FULL>
+__device__ __forceinline__ void reconcile_chunk(int i0, const Columns<V, U, Idx, FULL>& col, float* params, float* mom,
+                                                float* sq, const float4& gbar, const StepArgs& step,
+                                                float4 (&th)[CH], float4 (&bu)[CH], float4 (&sv)[CH],
+                                                const float4 (&gw)[CH], float4& tsum, float4& bsum, float4& ssum) {
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
-        if (i0 + k < W) {
+        if (i0 + k < col.W) {
             opt_step4<OPT>(METHOD == kMethodLocalSGD ? gw[k] : gbar, th[k], bu[k], sv[k], step);
             if (STATE_SYNC) {
                 add4(bsum, bu[k]);
                 if (OPT == kOptAdamW) add4(ssum, sv[k]);
             } else {
-                m4[CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq)] = bu[k];
-                if (OPT == kOptAdamW) s4[CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq)] = sv[k];
+                col.store(mom, (Idx)(i0 + k), bu[k]);
+                if (OPT == kOptAdamW) col.store(sq, (Idx)(i0 + k), sv[k]);
             }
             if (METHOD == kMethodDDP)
-                p4[CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq)] = th[k];
+                col.store(params, (Idx)(i0 + k), th[k]);
             else
                 add4(tsum, th[k]);
         }
     }
 }
 
+// SlowMo (eqs. 8-10) on 4 columns: the new velocity and the new model.
+__device__ __forceinline__ void slowmo4(const float4& avg, const float4& ref, const float4& vel, const SyncArgs& a,
+                                        float4& vn, float4& tn) {
+    vn.x = fmaf(a.beta, vel.x, avg.x - ref.x);
+    vn.y = fmaf(a.beta, vel.y, avg.y - ref.y);
+    vn.z = fmaf(a.beta, vel.z, avg.z - ref.z);
+    vn.w = fmaf(a.beta, vel.w, avg.w - ref.w);
+    tn.x = fmaf(a.alpha, vn.x, ref.x);
+    tn.y = fmaf(a.alpha, vn.y, ref.y);
+    tn.z = fmaf(a.alpha, vn.z, ref.z);
+    tn.w = fmaf(a.alpha, vn.w, ref.w);
+}
+
+// The whole reconcile of one thread's columns.
+template <int METHOD, int OPT, bool STATE_SYNC, typename G, int CH, bool LATE_ANCHOR, int GCH, bool OVERLAP, int V, int U,
+          typename Idx, bool FULL>
+__device__ __forceinline__ void reconcile_columns(const Columns<V, U, Idx, FULL>& col, float* __restrict__ params,
+                                                  float* __restrict__ mom, float* __restrict__ sq,
+                                                  const G* __restrict__ grads, float* __restrict__ anchor,
+                                                  float* __restrict__ slow_v, const SyncArgs& a) {
+    static_assert(!(STATE_SYNC && METHOD == kMethodDDP), "DDP's states are identical across workers");
+    static_assert(!(OVERLAP && METHOD == kMethodLocalSGD), "LocalSGD has no gradient mean to overlap");
+    const int W = col.W;
+    float4 ref, vel;
+    if (METHOD == kMethodCPDP && !LATE_ANCHOR) {
+        ref = col.load(anchor, 0, 1);
+        vel = col.load(slow_v, 0, 1);
+    }
+
+    // 1. gradient mean (eq. 2)
+    float4 gbar = make_float4(0.f, 0.f, 0.f, 0.f);
+    // the rows of the current state chunk (the first one loaded in step 1 when OVERLAP)
+    float4 th[CH], bu[CH], sv[CH];
+    if (METHOD != kMethodLocalSGD) {
+        float4 gsum = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (GCH == CH && !OVERLAP) {
+            for (int i0 = 0; i0 < W; i0 += CH) {
+                float4 gv[CH];
+#pragma unroll
+                for (int k = 0; k < CH; ++k)
+                    if (i0 + k < W) gv[k] = col.grads(grads, (Idx)(i0 + k));
+#pragma unroll
+                for (int k = 0; k < CH; ++k)
+                    if (i0 + k < W) add4(gsum, gv[k]);
+            }
+        } else {
+            for (int i0 = 0; i0 < W; i0 += GCH) {
+                typename GradLoad<G>::Words gv[GCH];
+#pragma unroll
+                for (int k = 0; k < GCH; ++k)
+                    if (i0 + k < W) gv[k] = col.words(grads, (Idx)(i0 + k));
+                if (OVERLAP && i0 == 0) {
+#pragma unroll
+                    for (int k = 0; k < CH; ++k) {
+                        if (k < W) {
+                            th[k] = col.load(params, (Idx)k);
+                            bu[k] = col.load(mom, (Idx)k);
+                            if (OPT == kOptAdamW) sv[k] = col.load(sq, (Idx)k);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < GCH; ++k)
+                    if (i0 + k < W) add4(gsum, GradLoad<G>::widen(gv[k]));
+            }
+        }
+        gbar = div4(gsum, a.workers);
+    }
+
+    // 2-3. optimizer step on every worker (eq. 6: with gbar; LocalSGD: with
+    // its own gradient), then the mean of the stepped replicas (eq. 7)
+    float4 tsum = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 bsum = make_float4(0.f, 0.f, 0.f, 0.f), ssum = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i0 = 0; i0 < W; i0 += CH) {
+        float4 gw[CH];
+        if (!(OVERLAP && i0 == 0)) {
+#pragma unroll
+            for (int k = 0; k < CH; ++k) {
+                if (i0 + k < W) {
+                    th[k] = col.load(params, (Idx)(i0 + k));
+                    bu[k] = col.load(mom, (Idx)(i0 + k));
+                    if (OPT == kOptAdamW) sv[k] = col.load(sq, (Idx)(i0 + k));
+                    if (METHOD == kMethodLocalSGD) gw[k] = col.grads(grads, (Idx)(i0 + k));
+                }
+            }
+        }
+        reconcile_chunk<METHOD, OPT, STATE_SYNC>(i0, col, params, mom, sq, gbar, a.step, th, bu, sv, gw, tsum, bsum, ssum);
+    }
+    if (METHOD == kMethodDDP) return;
+    if (STATE_SYNC) {
+        const float4 bmean = div4(bsum, a.workers);
+        for (int i = 0; i < W; ++i) col.store(mom, (Idx)i, bmean);
+        if (OPT == kOptAdamW) {
+            const float4 smean = div4(ssum, a.workers);
+            for (int i = 0; i < W; ++i) col.store(sq, (Idx)i, smean);
+        }
+    }
+    const float4 avg = div4(tsum, a.workers);
+
+    // 4. SlowMo (eqs. 8-10); LocalSGD writes the plain average
+    float4 tn = avg;
+    if (METHOD == kMethodCPDP) {
+        if (LATE_ANCHOR) {
+            ref = col.load(anchor, 0, 1);
+            vel = col.load(slow_v, 0, 1);
+        }
+        float4 vn;
+        slowmo4(avg, ref, vel, a, vn, tn);
+        col.store(anchor, 0, 1, tn);
+        col.store(slow_v, 0, 1, vn);
+    }
+
+    // 5. write-back to every replica (eqs. 11-12)
+    for (int i = 0; i < W; ++i) col.store(params, (Idx)i, tn);
+}
+
+// N a multiple of 4: one 128-bit vector per row and thread.
 template <int METHOD, int OPT, bool STATE_SYNC, typename G, int CH, int MIN_BLOCKS, bool LATE_ANCHOR, typename Idx,
           int GCH = CH, bool OVERLAP = false>
 __global__ void __launch_bounds__(kThreads, MIN_BLOCKS)
 reconcile_vec4_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
                       const G* __restrict__ grads, float* __restrict__ anchor, float* __restrict__ slow_v,
                       int W, Idx nq, SyncArgs a) {
-    static_assert(!(STATE_SYNC && METHOD == kMethodDDP), "DDP's states are identical across workers");
-    static_assert(!(OVERLAP && METHOD == kMethodLocalSGD), "LocalSGD has no gradient mean to overlap");
     pdl_wait_then_release();
-    float4* p4 = reinterpret_cast<float4*>(params);
-    float4* m4 = reinterpret_cast<float4*>(mom);
-    float4* s4 = reinterpret_cast<float4*>(sq);
-    float4* ref4 = reinterpret_cast<float4*>(anchor);
-    float4* vel4 = reinterpret_cast<float4*>(slow_v);
     for (Idx c = (Idx)blockIdx.x * blockDim.x + threadIdx.x; c < nq; c += (Idx)gridDim.x * blockDim.x) {
-        float4 ref, vel;
-        if (METHOD == kMethodCPDP && !LATE_ANCHOR) {
-            ref = ref4[CPDP_IDX(c, nq)];
-            vel = vel4[CPDP_IDX(c, nq)];
-        }
-
-        // 1. gradient mean (eq. 2)
-        float4 gbar = make_float4(0.f, 0.f, 0.f, 0.f);
-        // the rows of the current state chunk (the first one loaded in step 1 when OVERLAP)
-        float4 th[CH], bu[CH], sv[CH];
-        if (METHOD != kMethodLocalSGD) {
-            float4 gsum = make_float4(0.f, 0.f, 0.f, 0.f);
-            if constexpr (GCH == CH && !OVERLAP) {
-                for (int i0 = 0; i0 < W; i0 += CH) {
-                    float4 gv[CH];
-#pragma unroll
-                    for (int k = 0; k < CH; ++k)
-                        if (i0 + k < W) gv[k] = GradLoad<G>::vec4(grads, CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq));
-#pragma unroll
-                    for (int k = 0; k < CH; ++k)
-                        if (i0 + k < W) add4(gsum, gv[k]);
-                }
-            } else {
-                for (int i0 = 0; i0 < W; i0 += GCH) {
-                    typename GradLoad<G>::Words gv[GCH];
-#pragma unroll
-                    for (int k = 0; k < GCH; ++k)
-                        if (i0 + k < W) gv[k] = GradLoad<G>::words(grads, CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq));
-                    if (OVERLAP && i0 == 0) {
-#pragma unroll
-                        for (int k = 0; k < CH; ++k) {
-                            if (k < W) {
-                                th[k] = p4[CPDP_IDX((Idx)k * nq + c, (Idx)W * nq)];
-                                bu[k] = m4[CPDP_IDX((Idx)k * nq + c, (Idx)W * nq)];
-                                if (OPT == kOptAdamW) sv[k] = s4[CPDP_IDX((Idx)k * nq + c, (Idx)W * nq)];
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < GCH; ++k)
-                        if (i0 + k < W) add4(gsum, GradLoad<G>::widen(gv[k]));
-                }
-            }
-            gbar = div4(gsum, a.workers);
-        }
-
-        // 2-3. optimizer step on every worker (eq. 6: with gbar; LocalSGD: with
-        // its own gradient), then the mean of the stepped replicas (eq. 7)
-        float4 tsum = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 bsum = make_float4(0.f, 0.f, 0.f, 0.f), ssum = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int i0 = 0; i0 < W; i0 += CH) {
-            float4 gw[CH];
-            if (!(OVERLAP && i0 == 0)) {
-#pragma unroll
-                for (int k = 0; k < CH; ++k) {
-                    if (i0 + k < W) {
-                        th[k] = p4[CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq)];
-                        bu[k] = m4[CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq)];
-                        if (OPT == kOptAdamW) sv[k] = s4[CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq)];
-                        if (METHOD == kMethodLocalSGD) gw[k] = GradLoad<G>::vec4(grads, CPDP_IDX((Idx)(i0 + k) * nq + c, (Idx)W * nq));
-                    }
-                }
-            }
-            reconcile_chunk<METHOD, OPT, STATE_SYNC, CH, Idx>(i0, W, nq, c, p4, m4, s4, gbar, a.step, th, bu, sv, gw, tsum,
-                                                              bsum, ssum);
-        }
-        if (METHOD == kMethodDDP) continue;
-        if (STATE_SYNC) {
-            const float4 bmean = div4(bsum, a.workers);
-            for (int i = 0; i < W; ++i) m4[CPDP_IDX((Idx)i * nq + c, (Idx)W * nq)] = bmean;
-            if (OPT == kOptAdamW) {
-                const float4 smean = div4(ssum, a.workers);
-                for (int i = 0; i < W; ++i) s4[CPDP_IDX((Idx)i * nq + c, (Idx)W * nq)] = smean;
-            }
-        }
-        const float4 avg = div4(tsum, a.workers);
-
-        // 4. SlowMo (eqs. 8-10); LocalSGD writes the plain average
-        float4 tn = avg;
-        if (METHOD == kMethodCPDP) {
-            if (LATE_ANCHOR) {
-                ref = ref4[CPDP_IDX(c, nq)];
-                vel = vel4[CPDP_IDX(c, nq)];
-            }
-            float4 vn;
-            vn.x = fmaf(a.beta, vel.x, avg.x - ref.x);
-            vn.y = fmaf(a.beta, vel.y, avg.y - ref.y);
-            vn.z = fmaf(a.beta, vel.z, avg.z - ref.z);
-            vn.w = fmaf(a.beta, vel.w, avg.w - ref.w);
-            tn.x = fmaf(a.alpha, vn.x, ref.x);
-            tn.y = fmaf(a.alpha, vn.y, ref.y);
-            tn.z = fmaf(a.alpha, vn.z, ref.z);
-            tn.w = fmaf(a.alpha, vn.w, ref.w);
-            ref4[CPDP_IDX(c, nq)] = tn;
-            vel4[CPDP_IDX(c, nq)] = vn;
-        }
-
-        // 5. write-back to every replica (eqs. 11-12)
-        for (int i = 0; i < W; ++i) p4[CPDP_IDX((Idx)i * nq + c, (Idx)W * nq)] = tn;
+        const Columns<4, 1, Idx> col{nq, c, W};
+        reconcile_columns<METHOD, OPT, STATE_SYNC, G, CH, LATE_ANCHOR, GCH, OVERLAP>(col, params, mom, sq, grads,
+                                                                                    anchor, slow_v, a);
     }
 }
 
@@ -578,14 +699,7 @@ reconcile_onepass_kernel(float* __restrict__ params, float* __restrict__ mom, fl
         float4 tn = avg;
         if (METHOD == kMethodCPDP) {
             float4 vn;
-            vn.x = fmaf(a.beta, vel.x, avg.x - ref.x);
-            vn.y = fmaf(a.beta, vel.y, avg.y - ref.y);
-            vn.z = fmaf(a.beta, vel.z, avg.z - ref.z);
-            vn.w = fmaf(a.beta, vel.w, avg.w - ref.w);
-            tn.x = fmaf(a.alpha, vn.x, ref.x);
-            tn.y = fmaf(a.alpha, vn.y, ref.y);
-            tn.z = fmaf(a.alpha, vn.z, ref.z);
-            tn.w = fmaf(a.alpha, vn.w, ref.w);
+            slowmo4(avg, ref, vel, a, vn, tn);
             ref4[CPDP_IDX(c, nq)] = tn;
             vel4[CPDP_IDX(c, nq)] = vn;
         }
@@ -596,61 +710,27 @@ reconcile_onepass_kernel(float* __restrict__ params, float* __restrict__ mom, fl
     }
 }
 
-// Same computation, one parameter per thread, for any N (rows need not be
-// 16-byte aligned).
-template <int METHOD, int OPT, bool STATE_SYNC, typename G>
-__global__ void __launch_bounds__(kThreads)
+// Any other N: V = 2 elements at a time where N is even, else V = 1 (`units`
+// is N / V), U such units per thread. The sums run in the order of the vector
+// kernel's, so the results are bit-identical to it column by column.
+template <int METHOD, int OPT, bool STATE_SYNC, typename G, int V, int U, int CH, int MIN_BLOCKS, bool LATE_ANCHOR,
+          typename Idx, int GCH = CH, bool OVERLAP = false>
+__global__ void __launch_bounds__(kThreads, MIN_BLOCKS)
 reconcile_scalar_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
                         const G* __restrict__ grads, float* __restrict__ anchor, float* __restrict__ slow_v,
-                        int W, int64_t N, SyncArgs a) {
-    static_assert(!(STATE_SYNC && METHOD == kMethodDDP), "DDP's states are identical across workers");
+                        int W, Idx units, SyncArgs a) {
     pdl_wait_then_release();
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        float gbar = 0.f;
-        if (METHOD != kMethodLocalSGD) {
-            float gsum = 0.f;
-            for (int i = 0; i < W; ++i) gsum += GradLoad<G>::one(grads, CPDP_IDX((int64_t)i * N + j, (int64_t)W * N));
-            gbar = gsum / a.workers;
+    const Idx warp = ((Idx)blockIdx.x * blockDim.x + threadIdx.x) / 32;
+    for (Idx u = warp * (32 * U) + threadIdx.x % 32; u < units; u += (Idx)gridDim.x * blockDim.x * U) {
+        if (U == 1 || u - (Idx)(threadIdx.x % 32) + 32 * U <= units) {  // every column of the warp exists
+            const Columns<V, U, Idx, true> col{units, u, W};
+            reconcile_columns<METHOD, OPT, STATE_SYNC, G, CH, LATE_ANCHOR, GCH, OVERLAP>(col, params, mom, sq, grads,
+                                                                                        anchor, slow_v, a);
+        } else {
+            const Columns<V, U, Idx, false> col{units, u, W};
+            reconcile_columns<METHOD, OPT, STATE_SYNC, G, 1, true, 1, false>(col, params, mom, sq, grads, anchor,
+                                                                             slow_v, a);
         }
-        float tsum = 0.f, bsum = 0.f, ssum = 0.f;
-        for (int i = 0; i < W; ++i) {
-            float th = params[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)];
-            float bu = mom[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)];
-            float sv = 0.f;
-            if (OPT == kOptAdamW) sv = sq[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)];
-            const float g = METHOD == kMethodLocalSGD ? GradLoad<G>::one(grads, CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)) : gbar;
-            opt_step<OPT>(g, th, bu, sv, a.step);
-            if (STATE_SYNC) {
-                bsum += bu;
-                ssum += sv;
-            } else {
-                mom[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)] = bu;
-                if (OPT == kOptAdamW) sq[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)] = sv;
-            }
-            if (METHOD == kMethodDDP)
-                params[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)] = th;
-            else
-                tsum += th;
-        }
-        if (METHOD == kMethodDDP) continue;
-        if (STATE_SYNC) {
-            const float bmean = bsum / a.workers, smean = ssum / a.workers;
-            for (int i = 0; i < W; ++i) {
-                mom[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)] = bmean;
-                if (OPT == kOptAdamW) sq[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)] = smean;
-            }
-        }
-        const float avg = tsum / a.workers;
-        float tn = avg;
-        if (METHOD == kMethodCPDP) {
-            const float ref = anchor[CPDP_IDX(j, N)];
-            const float vn = fmaf(a.beta, slow_v[CPDP_IDX(j, N)], avg - ref);
-            tn = fmaf(a.alpha, vn, ref);
-            anchor[CPDP_IDX(j, N)] = tn;
-            slow_v[CPDP_IDX(j, N)] = vn;
-        }
-        for (int i = 0; i < W; ++i) params[CPDP_IDX((int64_t)i * N + j, (int64_t)W * N)] = tn;
     }
 }
 

@@ -210,6 +210,61 @@ struct GradChunkOf<S, std::void_t<decltype(S::grad_rows)>> {
     static constexpr bool overlap = S::overlap;
 };
 
+// N not a multiple of 4 (reconcile_scalar_kernel): V = 2 elements per load where
+// N is even, else 1. The row bytes are the same as for any N; what a
+// one-column-per-thread kernel lacks is bytes in flight per thread, and past
+// that the narrow loads cost instructions and, at odd N, a fifth 32-byte
+// sector per 128-byte row segment. So a thread owns 4 columns in 4 / V loads
+// (a warp covers kRaggedColumns of a row) and loads rows in chunks as the
+// vector kernel does. Sync-step GB/s at N = 23.7 M, W = 8, before (one column
+// per thread, one row at a time) and now, N odd / N = 2 mod 4: CPDP SGD f32
+// 5,264 -> 6,872 / 5,256 -> 7,039; SGD bf16 5,023 -> 6,422 / 5,000 -> 6,979;
+// AdamW f32 5,499 -> 6,725 / 5,488 -> 6,952; AdamW bf16 5,306 -> 6,493 /
+// 5,302 -> 6,938; with state reconciliation 6,040-6,504 -> 6,568-6,757 (SGD)
+// and 5,446-5,687 -> 6,430-6,909 (AdamW). Eight shapes were swept at W = 1 to
+// 16: gradient chunks overlapped with the first state chunk win where the loads
+// are pairs, and for SGD f32 at odd N; the other odd-N variants are
+// short of registers and take plain 2-row or 1-row chunks.
+constexpr int kRaggedColumns = 128;
+template <int V, int OPT, bool SS, typename G, bool MANY>
+struct RaggedShape {
+    static constexpr bool f32 = std::is_same<G, float>::value;
+    static constexpr bool overlap = V == 2 ? !(SS && OPT == kOptAdamW) : !SS && OPT == kOptSGD && f32;
+    static constexpr bool three = overlap && OPT == kOptAdamW && MANY;
+    static constexpr int rows = three ? 3 : V == 1 && SS && (OPT == kOptAdamW || f32) ? 1 : 2;
+    static constexpr int min_blocks = three ? 3 : 4;
+    static constexpr int grad_rows = !overlap ? rows : f32 ? 4 : 8;
+    static constexpr bool late = true;
+};
+
+// Few columns: at 4 columns per thread N = 300,000 gives an SM two of the four
+// blocks it can hold, so up to kRaggedNarrowColumns a thread owns one load's
+// columns instead and 4-row chunks keep it busy (W = 8, N = 100,001, us, one
+// column and one row at a time / 4 columns / this: CPDP SGD f32 5.15 / 5.87 /
+// 4.29; N = 300,002 AdamW bf16 15.1 / 16.2 / 12.7). The lines are where the two
+// cross (SGD f32 at W = 8: N = 300,001 12.4 narrow, 11.6 wide; N = 300,002 10.3
+// and 11.8; N = 600,002 18.7 and 17.8; AdamW f32 at N = 600,002 25.0 and 30.9,
+// at 2,000,002 76.5 and 75.5). State-reconciling SGD stores nothing inside its
+// row loop, so the compiler overlaps its 1-row chunks by itself.
+template <int V, int OPT, bool SS>
+constexpr int64_t kRaggedNarrowColumns = V == 2 ? (OPT == kOptAdamW || SS ? 1'500'000 : 500'000)
+                                                : (OPT == kOptAdamW ? 400'000 : 200'000);
+template <int V, int OPT, bool SS, typename G>
+struct RaggedShapeNarrow {
+    static constexpr bool overlap = !(SS && OPT == kOptSGD);
+    static constexpr int rows = overlap ? 4 : 1, min_blocks = overlap || V == 2 ? 4 : 6;
+    static constexpr int grad_rows = !overlap ? 1 : std::is_same<G, float>::value ? 4 : 8;
+    static constexpr bool late = true;
+};
+
+// One worker: all rows of a column in one round trip (N = 23.7 M, SGD f32
+// 4,244 -> 6,681 GB/s at odd N, 4,251 -> 6,656 at N = 2 mod 4; AdamW bf16
+// 4,579 -> 6,609 and 4,582 -> 6,616).
+struct RaggedShapeW1 {
+    static constexpr int rows = 1, min_blocks = 4, grad_rows = 1;
+    static constexpr bool late = false, overlap = true;
+};
+
 // One round trip for few workers (reconcile_onepass_kernel: every row of a
 // column loaded before any is used). Where it is used, and at how many
 // resident blocks, per method, optimizer, state reconciliation and gradient
