@@ -296,6 +296,7 @@ cpdp_status cpdp_set_reconcile_shuffle(cpdp_ctx *ctx, int enable);
  * reconcile on ctx launched (cpdp_reconcile, or a reconcile step of
  * cpdp_step, cpdp_step_at or the host-fed calls): "reconcile_vec4_kernel",
  * "reconcile_onepass_kernel", "reconcile_scalar_kernel",
+ * "reconcile_split_kernel" (many workers over few columns),
  * "reconcile_tma_kernel" or "reconcile_shuffle_kernel"; "" before the first
  * one. The launch shape is chosen per worker count, method, optimizer, state
  * reconciliation and gradient type, so this tells a caller (a profile, a

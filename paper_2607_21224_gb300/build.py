@@ -14,9 +14,10 @@ PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
 INCLUDE = ROOT / "include"
 CSRC = PKG / "csrc"
-SOURCES = [CSRC / "cpdp.cu", CSRC / "cpdp_ragged.cu"]
+SOURCES = [CSRC / "cpdp.cu", CSRC / "cpdp_ragged.cu", CSRC / "cpdp_split.cu"]
 DEPENDS = SOURCES + [CSRC / "cpdp_kernels.cuh", CSRC / "cpdp_shapes.cuh", CSRC / "cpdp_tma.cuh",
-                     CSRC / "cpdp_floor.cuh", CSRC / "cpdp_shuffle.cuh", CSRC / "cpdp_launch.cuh", INCLUDE / "cpdp.h"]
+                     CSRC / "cpdp_floor.cuh", CSRC / "cpdp_shuffle.cuh", CSRC / "cpdp_split.cuh",
+                     CSRC / "cpdp_launch.cuh", INCLUDE / "cpdp.h"]
 LIBRARY = PKG / "libcpdp.so"
 CHECKED_LIBRARY = PKG / "libcpdp_checked.so"  # debug build: kernels count out-of-range indices
 BUILD_DIR = ROOT / "_build"

@@ -9,6 +9,7 @@
 #include "cpdp_launch.cuh"
 #include "cpdp_shapes.cuh"
 #include "cpdp_shuffle.cuh"
+#include "cpdp_split.cuh"
 #include "cpdp_tma.cuh"
 
 #include <cmath>
@@ -283,6 +284,13 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
     const cpdp::SyncArgs a{step, c->beta, c->alpha, static_cast<float>(c->W)};
     float* sq = OPT == cpdp::kOptAdamW ? c->exp_avg_sq : nullptr;
     const G* g = static_cast<const G*>(grads);
+    // what the kernels of the other translation units take
+    const cpdp::ReconcileCall call{c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
+                                   c->anchor, c->slow_v, a, s};
+    if (cpdp::split_takes(c->W, c->N)) {
+        c->reconcile_kernel = "reconcile_split_kernel";
+        return cpdp::launch_reconcile_split(call);
+    }
     if ((c->N & 3) == 0) {
         const int64_t nq = c->N >> 2;
         // few workers: one round trip where it measured faster (cpdp_shapes.cuh)
@@ -318,8 +326,7 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
         return launch_vec4<cpdp::ReconcileShape<OPT, G, SS>, METHOD, OPT, SS, G>(c, g, sq, s, a, nq);
     }
     c->reconcile_kernel = "reconcile_scalar_kernel";
-    return cpdp::launch_reconcile_ragged({c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
-                                          c->anchor, c->slow_v, a, s});
+    return cpdp::launch_reconcile_ragged(call);
 }
 
 template <int METHOD, int OPT, typename G>
@@ -958,10 +965,11 @@ cpdp_status cpdp_bad_index_count(cpdp_ctx* ctx, int64_t* count) {
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpyFromSymbol(&seen, cpdp::bad_index_count, sizeof seen);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(cpdp::bad_index_count, &zero, sizeof zero);
-    unsigned long long ragged = 0;  // the other translation unit's own counter
+    unsigned long long ragged = 0, split = 0;  // the other translation units' own counters
     if (e == cudaSuccess) e = cpdp::take_bad_indices_ragged(&ragged);
+    if (e == cudaSuccess) e = cpdp::take_bad_indices_split(&split);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "reading the bad-index count");
-    *count = static_cast<int64_t>(seen + ragged);
+    *count = static_cast<int64_t>(seen + ragged + split);
 #else
     *count = -1;  // a release build checks no index
 #endif

@@ -47,6 +47,8 @@ struct ReconcileCall {
 
 // N not a multiple of 4 (cpdp_ragged.cu).
 cudaError_t launch_reconcile_ragged(const ReconcileCall& c);
+// Many workers over few columns (cpdp_split.cu).
+cudaError_t launch_reconcile_split(const ReconcileCall& c);
 
 // The call's variant as compile-time constants: f.template run<METHOD, OPT, SS, G>().
 template <typename F, int METHOD, int OPT, bool SS>
@@ -73,5 +75,6 @@ cudaError_t dispatch_reconcile(const ReconcileCall& c, const F& f) {
 // The index-checked debug build counts bad indices per translation unit; each
 // file's counter, read and set to 0 (current device, after a synchronization).
 cudaError_t take_bad_indices_ragged(unsigned long long* count);
+cudaError_t take_bad_indices_split(unsigned long long* count);
 
 }  // namespace cpdp

@@ -1,0 +1,254 @@
+// The reconcile with the worker rows of a column split across the warps of a
+// block, for many workers over few columns.
+//
+// What bounds the column kernels there: one thread walks all W rows of its
+// columns, a chunk at a time, so a launch takes about W / 2 dependent trips to
+// memory however few columns there are, and N / 1024 blocks cannot fill 152
+// SMs (W = 64, N = 60,000: 59 blocks, 32.8 us for 78 MB). Here a block owns 32 loads' columns
+// (64 at even N, 32 at odd) and its 4 to 16 warps take every R-th row, so a
+// column's rows are loaded by R warps at once and N / 64 blocks run. The
+// values to be averaged pass through shared memory, where one thread per
+// column adds them in worker order: the sums are those of the other kernels
+// bit for bit (partial sums per warp measured the same within 10 %, but in
+// another order). Sync step, us, column kernels -> this one, CPDP SGD f32: W = 64,
+// N = 60,000 32.8 -> 15.6 (5.0 TB/s; the bytes take 11.4 at the copy rate);
+// W = 16, N = 20,000 5.54 -> 2.26; W = 200, N = 20,000 90.6 -> 22.9; AdamW bf16
+// W = 64, N = 20,000 4.5 times as fast.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "cpdp_kernels.cuh"
+
+namespace cpdp {
+
+constexpr int kSplitMaxWarps = 16;
+
+// Where it is used. From 9 workers: up to 8 the column kernels need at most
+// four trips. Above these sizes the column kernels have blocks enough, and
+// their longer row segments win (ratio of sync-step times, column kernel over
+// this one): even N, W = 9: N = 60,000 1.17-1.40 for SGD, 100,000 0.85-1.18;
+// W = 16: 100,000 1.04-1.61, 200,000 0.85-1.24; W = 64: 100,000 1.26-1.72,
+// 200,000 1.04-1.27, 400,000 0.92-1.02. Odd N, W = 9: 20,001 1.24-1.32,
+// 60,001 0.79-0.85; W = 24: 60,001 1.11-1.25, 100,001 0.87-1.02; W = 64:
+// 60,001 1.27-1.44, 100,001 1.01-1.15.
+inline bool split_takes(int W, int64_t N) {
+    if (W < 9) return false;
+    if ((N & 1) == 0) return N <= (W < 16 ? 64'000 : 160'000);
+    return N <= (W < 24 ? 24'000 : 64'000);
+}
+
+// Warps per block over `tiles` blocks: more while the launch stays within
+// about one resident wave (152 SMs x 28 warps) and a warp keeps 3 rows or more
+// (CPDP SGD f32 with partial sums, us at 4 / 8 / 16 warps: W = 16, N = 32,000
+// 2.47 / 3.29 / -; W = 64, N = 32,000 10.9 / 9.5 / -; W = 200, N = 8,000 21.4 /
+// 13.7 / 11.4).
+inline int split_warps(int W, int64_t tiles) {
+    int warps = 4;
+    while (warps < kSplitMaxWarps && tiles * warps * 2 <= 4096 && W >= 3 * warps * 2) warps *= 2;
+    return warps;
+}
+
+// V consecutive columns of one row.
+template <int V>
+struct Slice {
+    float v[V];
+};
+
+template <int V>
+struct SliceIO;
+template <>
+struct SliceIO<2> {
+    static __device__ __forceinline__ Slice<2> load(const float* p, int32_t u) {
+        const float2 x = reinterpret_cast<const float2*>(p)[u];
+        return {x.x, x.y};
+    }
+    static __device__ __forceinline__ void store(float* p, int32_t u, const Slice<2>& x) {
+        reinterpret_cast<float2*>(p)[u] = make_float2(x.v[0], x.v[1]);
+    }
+    static __device__ __forceinline__ float2 words(const float* g, int32_t u) {
+        float2 x;
+        GradLoad<float>::pair(g, u, x.x, x.y);
+        return x;
+    }
+    static __device__ __forceinline__ uint32_t words(const bf16_bits* g, int32_t u) {
+        return GradLoad<bf16_bits>::pair(g, u);
+    }
+    static __device__ __forceinline__ Slice<2> widen(const float2& x) { return {x.x, x.y}; }
+    static __device__ __forceinline__ Slice<2> widen(uint32_t x) {
+        return {__uint_as_float(x << 16), __uint_as_float(x & 0xffff0000u)};
+    }
+};
+template <>
+struct SliceIO<1> {
+    static __device__ __forceinline__ Slice<1> load(const float* p, int32_t u) { return {p[u]}; }
+    static __device__ __forceinline__ void store(float* p, int32_t u, const Slice<1>& x) { p[u] = x.v[0]; }
+    template <typename G>
+    static __device__ __forceinline__ float words(const G* g, int32_t u) {
+        return GradLoad<G>::one(g, u);
+    }
+    static __device__ __forceinline__ Slice<1> widen(float x) { return {x}; }
+};
+
+// Rows of one round: their values pass through shared memory, where one
+// thread per column adds them in worker order.
+template <bool STATE_SYNC>
+struct SplitRows {
+    static constexpr int value = STATE_SYNC ? 32 : 64;
+};
+
+// s + rows[0][column] + ... + rows[n - 1][column], in that order.
+template <int C>
+__device__ __forceinline__ float add_rows(float s, const float (*rows)[C], int n, int column) {
+#pragma unroll 8
+    for (int r = 0; r < n; ++r) s += rows[r][column];
+    return s;
+}
+
+// A block owns C = 32 * V columns; its warp w of R takes rows w, w + R, ... of
+// them. `units` is N / V.
+template <int METHOD, int OPT, bool STATE_SYNC, typename G, int V, int CH, int GCH>
+__global__ void __launch_bounds__(32 * kSplitMaxWarps, 2)
+reconcile_split_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
+                       const G* __restrict__ grads, float* __restrict__ anchor, float* __restrict__ slow_v,
+                       int W, int32_t units, SyncArgs a) {
+    static_assert(!(STATE_SYNC && METHOD == kMethodDDP), "DDP's states are identical across workers");
+    using IO = SliceIO<V>;
+    constexpr int C = 32 * V, B = SplitRows<STATE_SYNC>::value;
+    __shared__ __align__(8) float rows_t[B][C];  // the gradients, then the stepped parameters
+    __shared__ __align__(8) float rows_b[STATE_SYNC ? B : 1][C];
+    __shared__ __align__(8) float rows_s[STATE_SYNC && OPT == kOptAdamW ? B : 1][C];
+    __shared__ __align__(8) float mean[3][C];  // what the columns' threads hand back to the warps
+    pdl_wait_then_release();
+    const int R = blockDim.x / 32, w = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int32_t u = (int32_t)blockIdx.x * 32 + lane;
+    const bool in = u < units;  // lanes past the last column only take part in the barriers
+    // the thread that adds column t of the block
+    const int t = threadIdx.x;
+    const int32_t column = (int32_t)blockIdx.x * C + t, columns = units * V;
+    const bool adds = t < C && column < columns;
+    auto at = [&](int row) { return CPDP_IDX(row * units + u, W * units); };
+    auto put = [&](float (*rows)[C], int r, const Slice<V>& x) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) rows[r][lane * V + e] = x.v[e];
+    };
+    auto get = [&](const float* row) {
+        Slice<V> x;
+#pragma unroll
+        for (int e = 0; e < V; ++e) x.v[e] = row[lane * V + e];
+        return x;
+    };
+
+    Slice<V> th[CH], bu[CH], sv[CH], gw[CH];
+    auto load_state = [&](int i0, int end) {
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            const int row = i0 + k * R;
+            if (in && row < end) {
+                th[k] = IO::load(params, at(row));
+                bu[k] = IO::load(mom, at(row));
+                if (OPT == kOptAdamW) sv[k] = IO::load(sq, at(row));
+                if (METHOD == kMethodLocalSGD) gw[k] = IO::widen(IO::words(grads, at(row)));
+            }
+        }
+    };
+    load_state(w, min(B, W));
+    float ref = 0.f, vel = 0.f;
+    if (METHOD == kMethodCPDP && adds) {
+        ref = anchor[CPDP_IDX(column, columns)];
+        vel = slow_v[CPDP_IDX(column, columns)];
+    }
+
+    // 1. gradient mean (eq. 2)
+    Slice<V> gbar = {};
+    if (METHOD != kMethodLocalSGD) {
+        float gsum = 0.f;
+        for (int base = 0; base < W; base += B) {
+            const int end = min(base + B, W);
+            for (int i0 = base + w; i0 < end; i0 += GCH * R) {
+                decltype(IO::words(grads, 0)) gv[GCH];
+#pragma unroll
+                for (int k = 0; k < GCH; ++k)
+                    if (in && i0 + k * R < end) gv[k] = IO::words(grads, at(i0 + k * R));
+#pragma unroll
+                for (int k = 0; k < GCH; ++k)
+                    if (in && i0 + k * R < end) put(rows_t, i0 + k * R - base, IO::widen(gv[k]));
+            }
+            __syncthreads();
+            if (adds) gsum = add_rows<C>(gsum, rows_t, end - base, t);
+            if (end == W && t < C) mean[0][t] = gsum / a.workers;
+            __syncthreads();
+        }
+        gbar = get(mean[0]);
+    }
+
+    // 2-3. optimizer step on the warp's workers (eq. 6), and the mean of the stepped replicas (eq. 7)
+    float tsum = 0.f, bsum = 0.f, ssum = 0.f;
+    for (int base = 0; base < W; base += B) {
+        const int end = min(base + B, W);
+        for (int i0 = base + w; i0 < end; i0 += CH * R) {
+            if (i0 != w) load_state(i0, end);
+#pragma unroll
+            for (int k = 0; k < CH; ++k) {
+                const int row = i0 + k * R;
+                if (in && row < end) {
+#pragma unroll
+                    for (int e = 0; e < V; ++e)
+                        opt_step<OPT>(METHOD == kMethodLocalSGD ? gw[k].v[e] : gbar.v[e], th[k].v[e], bu[k].v[e],
+                                      sv[k].v[e], a.step);
+                    if (STATE_SYNC) {
+                        put(rows_b, row - base, bu[k]);
+                        if (OPT == kOptAdamW) put(rows_s, row - base, sv[k]);
+                    } else {
+                        IO::store(mom, at(row), bu[k]);
+                        if (OPT == kOptAdamW) IO::store(sq, at(row), sv[k]);
+                    }
+                    if (METHOD == kMethodDDP)
+                        IO::store(params, at(row), th[k]);
+                    else
+                        put(rows_t, row - base, th[k]);
+                }
+            }
+        }
+        if (METHOD == kMethodDDP) continue;
+        __syncthreads();
+        if (adds) {
+            tsum = add_rows<C>(tsum, rows_t, end - base, t);
+            if (STATE_SYNC) {
+                bsum = add_rows<C>(bsum, rows_b, end - base, t);
+                if (OPT == kOptAdamW) ssum = add_rows<C>(ssum, rows_s, end - base, t);
+            }
+            if (end == W) {
+                float tn = tsum / a.workers;
+                if (METHOD == kMethodCPDP) {  // 4. SlowMo (eqs. 8-10)
+                    const float vn = fmaf(a.beta, vel, tn - ref);
+                    tn = fmaf(a.alpha, vn, ref);
+                    anchor[CPDP_IDX(column, columns)] = tn;
+                    slow_v[CPDP_IDX(column, columns)] = vn;
+                }
+                mean[0][t] = tn;
+                if (STATE_SYNC) {
+                    mean[1][t] = bsum / a.workers;
+                    if (OPT == kOptAdamW) mean[2][t] = ssum / a.workers;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    if (METHOD == kMethodDDP || !in) return;
+
+    // 5. write-back to every replica (eqs. 11-12), and of the averaged state
+    const Slice<V> tn = get(mean[0]);
+    for (int i = w; i < W; i += R) IO::store(params, at(i), tn);
+    if (STATE_SYNC) {
+        const Slice<V> bmean = get(mean[1]);
+        for (int i = w; i < W; i += R) IO::store(mom, at(i), bmean);
+        if (OPT == kOptAdamW) {
+            const Slice<V> smean = get(mean[2]);
+            for (int i = w; i < W; i += R) IO::store(sq, at(i), smean);
+        }
+    }
+}
+
+}  // namespace cpdp

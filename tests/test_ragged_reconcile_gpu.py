@@ -32,7 +32,7 @@ def _arrays(st):
     return [x for x in (st.params, st.mom, st.anchor, st.slow_v, getattr(st, "exp_avg_sq", None)) if x is not None]
 
 
-@pytest.mark.parametrize("W", [1, 3, 8, 9])
+@pytest.mark.parametrize("W", [1, 3, 7, 8])
 @pytest.mark.parametrize("N", [2, 31, 33, 62, 66, 127, 130, 255, 1022, 1025, 3 * 1024 + 126, 200_001, 400_003, 500_002,
                                700_002, 1_500_002])
 def test_ragged_columns_match_the_vector_kernel(N, W):
