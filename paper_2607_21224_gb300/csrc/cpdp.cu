@@ -57,6 +57,7 @@ struct cpdp_ctx {
     float* exp_avg_sq = nullptr;  // caller-owned [W][N], AdamW second moments
     int64_t opt_step = 0;         // optimizer steps taken (AdamW bias correction)
     bool state_sync = false;      // optimizer-state reconciliation variant
+    int backwards = 0;            // the next launch's walk direction (alternates)
     bool pdl = true;              // programmatic dependent launches (cpdp_set_pdl)
     // reconcile rows staged through shared memory by bulk copies (cpdp_set_reconcile_staging):
     // 0 = off (direct loads), else the ring's slot count, with the launch's shared memory and grid
@@ -233,6 +234,9 @@ cpdp_status check_grads(cpdp_ctx* ctx, const void* grads, cpdp_dtype dtype) {
     return CPDP_OK;
 }
 
+// The walk direction of the launch being made; the next one goes the other way.
+int turn(cpdp_ctx* c) { return c->backwards ^= 1; }
+
 template <typename G>
 cudaError_t launch_local(cpdp_ctx* c, const void* grads, cudaStream_t s, const cpdp::StepArgs& a) {
     const int64_t total = static_cast<int64_t>(c->W) * c->N;
@@ -243,10 +247,10 @@ cudaError_t launch_local(cpdp_ctx* c, const void* grads, cudaStream_t s, const c
         return launch(c,
                       cpdp::local_step_kernel<cpdp::kOptAdamW, G, cpdp::kLocalUnroll,
                                               cpdp::LocalWarpRuns<cpdp::kOptAdamW, G>::value>,
-                      grid, s, c->params, c->mom, c->exp_avg_sq, g, total, a);
+                      grid, s, c->params, c->mom, c->exp_avg_sq, g, total, a, turn(c));
     return launch(c,
                   cpdp::local_step_kernel<cpdp::kOptSGD, G, cpdp::kLocalUnroll, cpdp::LocalWarpRuns<cpdp::kOptSGD, G>::value>,
-                  grid, s, c->params, c->mom, static_cast<float*>(nullptr), g, total, a);
+                  grid, s, c->params, c->mom, static_cast<float*>(nullptr), g, total, a, turn(c));
 }
 
 // The one-pass reconcile for at most Shape::wmax workers.
@@ -255,7 +259,7 @@ cudaError_t launch_onepass(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, c
     static_assert(Shape::use, "a one-pass shape that is not used");
     c->reconcile_kernel = "reconcile_onepass_kernel";
     return launch(c, cpdp::reconcile_onepass_kernel<METHOD, OPT, SS, G, Shape::wmax, Shape::min_blocks>,
-                  cpdp::grid_for(nq, cpdp::kThreads), s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a);
+                  cpdp::grid_for(nq, cpdp::kThreads), s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
 }
 
 // The vectorised reconcile in launch shape Shape, with 32-bit offsets where
@@ -271,12 +275,12 @@ cudaError_t launch_vec4(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, cons
             return launch(c,
                           cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks, Shape::late,
                                                       int32_t, grad_rows, overlap>,
-                          grid, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, static_cast<int32_t>(nq), a);
+                          grid, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, static_cast<int32_t>(nq), a, turn(c));
     }
     return launch(c,
                   cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks, Shape::late, int64_t,
                                               grad_rows, overlap>,
-                  grid, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a);
+                  grid, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
 }
 
 template <int METHOD, int OPT, bool SS, typename G>
@@ -285,8 +289,8 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
     float* sq = OPT == cpdp::kOptAdamW ? c->exp_avg_sq : nullptr;
     const G* g = static_cast<const G*>(grads);
     // what the kernels of the other translation units take
-    const cpdp::ReconcileCall call{c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
-                                   c->anchor, c->slow_v, a, s};
+    cpdp::ReconcileCall call{c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
+                                   c->anchor, c->slow_v, a, 0, s};
     if (cpdp::split_takes(c->W, c->N)) {
         c->reconcile_kernel = "reconcile_split_kernel";
         return cpdp::launch_reconcile_split(call);
@@ -326,6 +330,7 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
         return launch_vec4<cpdp::ReconcileShape<OPT, G, SS>, METHOD, OPT, SS, G>(c, g, sq, s, a, nq);
     }
     c->reconcile_kernel = "reconcile_scalar_kernel";
+    call.backwards = turn(c);
     return cpdp::launch_reconcile_ragged(call);
 }
 

@@ -42,6 +42,7 @@ struct ReconcileCall {
     const void* grads;
     float *anchor, *slow_v;
     SyncArgs args;
+    int backwards;
     cudaStream_t stream;
 };
 

@@ -20,7 +20,7 @@ cudaError_t launch_shape(const ReconcileCall& c) {
                          reconcile_scalar_kernel<METHOD, OPT, SS, G, V, U, Shape::rows, Shape::min_blocks, Shape::late, Idx,
                                                  Shape::grad_rows, Shape::overlap && METHOD != kMethodLocalSGD>,
                          grid, kThreads, 0, c.stream, c.params, c.mom, c.sq, static_cast<const G*>(c.grads), c.anchor,
-                         c.slow_v, c.W, static_cast<Idx>(units), c.args);
+                         c.slow_v, c.W, static_cast<Idx>(units), c.args, c.backwards);
 }
 
 struct Ragged {
