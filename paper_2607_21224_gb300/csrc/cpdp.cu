@@ -291,7 +291,7 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
     // what the kernels of the other translation units take
     cpdp::ReconcileCall call{c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
                                    c->anchor, c->slow_v, a, 0, s};
-    if (cpdp::split_takes(c->W, c->N)) {
+    if (cpdp::split_takes(call)) {
         c->reconcile_kernel = "reconcile_split_kernel";
         return cpdp::launch_reconcile_split(call);
     }

@@ -242,13 +242,15 @@ struct RaggedShape {
 // columns instead and 4-row chunks keep it busy (W = 8, N = 100,001, us, one
 // column and one row at a time / 4 columns / this: CPDP SGD f32 5.15 / 5.87 /
 // 4.29; N = 300,002 AdamW bf16 15.1 / 16.2 / 12.7). The lines are where the two
-// cross (SGD f32 at W = 8: N = 300,001 12.4 narrow, 11.6 wide; N = 300,002 10.3
+// cross (SGD f32, W = 64: the wide shape takes 62.1 us at N = 200,001, where it
+// fills SMs unevenly, the narrow one 41.1 at 150,001; W = 8: N = 300,001 12.4
+// narrow, 11.6 wide; N = 300,002 10.3
 // and 11.8; N = 600,002 18.7 and 17.8; AdamW f32 at N = 600,002 25.0 and 30.9,
 // at 2,000,002 76.5 and 75.5). State-reconciling SGD stores nothing inside its
 // row loop, so the compiler overlaps its 1-row chunks by itself.
 template <int V, int OPT, bool SS>
 constexpr int64_t kRaggedNarrowColumns = V == 2 ? (OPT == kOptAdamW || SS ? 1'500'000 : 500'000)
-                                                : (OPT == kOptAdamW ? 400'000 : 200'000);
+                                                : (OPT == kOptAdamW ? 400'000 : 250'000);
 template <int V, int OPT, bool SS, typename G>
 struct RaggedShapeNarrow {
     static constexpr bool overlap = !(SS && OPT == kOptSGD);

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "cpdp_kernels.cuh"
+#include "cpdp_launch.cuh"
 
 namespace cpdp {
 
@@ -33,10 +34,18 @@ constexpr int kSplitMaxWarps = 16;
 // 200,000 1.04-1.27, 400,000 0.92-1.02. Odd N, W = 9: 20,001 1.24-1.32,
 // 60,001 0.79-0.85; W = 24: 60,001 1.11-1.25, 100,001 0.87-1.02; W = 64:
 // 60,001 1.27-1.44, 100,001 1.01-1.15.
-inline bool split_takes(int W, int64_t N) {
-    if (W < 9) return false;
-    if ((N & 1) == 0) return N <= (W < 16 ? 64'000 : 160'000);
-    return N <= (W < 24 ? 24'000 : 64'000);
+// Odd rows cost the column kernels more with float32 gradients and no velocity
+// to update: DDP SGD f32 1.05-1.94 up to N = 300,001 at any W from 9 (W = 64, N = 100,001 39.2 ->
+// 28.6 us); LocalSGD and AdamW f32 from 16 workers 1.02-1.20 at 100,001 and 0.88-1.04 at
+// 150,001.
+inline bool split_takes(const ReconcileCall& c) {
+    if (c.W < 9) return false;
+    if ((c.N & 1) == 0) return c.N <= (c.W < 16 ? 64'000 : 160'000);
+    if (!c.bf16 && !c.state_sync) {
+        if (c.method == kMethodDDP && c.opt == kOptSGD) return c.N <= 300'000;
+        if ((c.method != kMethodCPDP || c.opt == kOptAdamW) && c.W >= 16) return c.N <= 110'000;
+    }
+    return c.N <= (c.W < 24 ? 24'000 : 64'000);
 }
 
 // Warps per block over `tiles` blocks: more while the launch stays within

@@ -31,7 +31,9 @@ def _match(W, N, wide, want):
                 for step in ("local_step", "reconcile"):
                     getattr(a, step)(g[:, :N].to(dtype).contiguous())
                     getattr(b, step)(g.to(dtype))
-            assert a.reconcile_kernel() == want
+            f32_rule = dtype == torch.float32 and not state_sync and (
+                (method, opt) == ("ddp", "sgd") or ((method, opt) != ("cpdp", "sgd") and W >= 16 and N <= 110_000))
+            assert a.reconcile_kernel() == (want or ("reconcile_split_kernel" if f32_rule else "reconcile_scalar_kernel"))
             assert b.reconcile_kernel() in ("reconcile_vec4_kernel", "reconcile_onepass_kernel")
             for x, y in zip(_arrays(a), _arrays(b)):
                 assert torch.equal(x, y[..., :N]), (method, opt, state_sync, dtype)
@@ -45,9 +47,8 @@ def test_split_rows_match_the_column_kernels(N, W):
 
 @pytest.mark.parametrize("W,N,want", [
     (8, 1200, "reconcile_vec4_kernel"), (9, 64_000, "reconcile_split_kernel"), (9, 64_004, "reconcile_vec4_kernel"),
-    (16, 160_000, "reconcile_split_kernel"), (23, 24_001, "reconcile_scalar_kernel"),
-    (24, 63_999, "reconcile_split_kernel"), (24, 64_001, "reconcile_scalar_kernel"),
-    (4096, 66, "reconcile_split_kernel")])
+    (16, 160_000, "reconcile_split_kernel"), (23, 24_001, None), (24, 63_999, "reconcile_split_kernel"),
+    (24, 64_001, None), (9, 159_999, None), (4096, 66, "reconcile_split_kernel")])
 def test_the_rule_that_selects_it(W, N, want):
     if W * WIDE > 1 << 26:  # 4,096 workers: a wider problem of its own size
         gen = torch.Generator(device="cuda").manual_seed(1)
