@@ -50,7 +50,8 @@ struct Ragged {
     }
     template <int METHOD, int OPT, bool SS, typename G>
     cudaError_t run() const {
-        return (c.N & 1) == 0 ? shaped<METHOD, OPT, SS, G, 2>() : shaped<METHOD, OPT, SS, G, 1>();
+        const bool singles = SS && OPT == kOptSGD && c.W > 1 && c.N <= kRaggedSinglesColumns;
+        return (c.N & 1) == 0 && !singles ? shaped<METHOD, OPT, SS, G, 2>() : shaped<METHOD, OPT, SS, G, 1>();
     }
 };
 

@@ -247,14 +247,18 @@ struct RaggedShape {
 // narrow, 11.6 wide; N = 300,002 10.3
 // and 11.8; N = 600,002 18.7 and 17.8; AdamW f32 at N = 600,002 25.0 and 30.9,
 // at 2,000,002 76.5 and 75.5). State-reconciling SGD stores nothing inside its
-// row loop, so the compiler overlaps its 1-row chunks by itself.
+// row loop and holds little per column, so 1-row chunks at 8 blocks of single
+// columns are as good as any up to 700,000 odd columns (W = 8, N = 300,001
+// 10.4 us; at 6 blocks 12.0, 4-row chunks 12.4) and beat pairs up to
+// kRaggedSinglesColumns even ones (W = 4, N = 100,002 2.5 us against 2.8).
+constexpr int64_t kRaggedSinglesColumns = 200'000;
 template <int V, int OPT, bool SS>
 constexpr int64_t kRaggedNarrowColumns = V == 2 ? (OPT == kOptAdamW || SS ? 1'500'000 : 500'000)
-                                                : (OPT == kOptAdamW ? 400'000 : 250'000);
+                                                : (OPT == kOptAdamW ? 400'000 : SS ? 700'000 : 250'000);
 template <int V, int OPT, bool SS, typename G>
 struct RaggedShapeNarrow {
     static constexpr bool overlap = !(SS && OPT == kOptSGD);
-    static constexpr int rows = overlap ? 4 : 1, min_blocks = overlap || V == 2 ? 4 : 6;
+    static constexpr int rows = overlap ? 4 : 1, min_blocks = overlap || V == 2 ? 4 : 8;
     static constexpr int grad_rows = !overlap ? 1 : std::is_same<G, float>::value ? 4 : 8;
     static constexpr bool late = true;
 };
