@@ -246,11 +246,13 @@ cudaError_t launch_local(cpdp_ctx* c, const void* grads, cudaStream_t s, const c
     if (c->optimizer == CPDP_OPT_ADAMW)
         return launch(c,
                       cpdp::local_step_kernel<cpdp::kOptAdamW, G, cpdp::kLocalUnroll,
-                                              cpdp::LocalWarpRuns<cpdp::kOptAdamW, G>::value>,
+                                              cpdp::LocalWarpRuns<cpdp::kOptAdamW, G>::value, false>,
                       grid, s, c->params, c->mom, c->exp_avg_sq, g, total, a, turn(c));
-    return launch(c,
-                  cpdp::local_step_kernel<cpdp::kOptSGD, G, cpdp::kLocalUnroll, cpdp::LocalWarpRuns<cpdp::kOptSGD, G>::value>,
-                  grid, s, c->params, c->mom, static_cast<float*>(nullptr), g, total, a, turn(c));
+    constexpr bool warp_runs = cpdp::LocalWarpRuns<cpdp::kOptSGD, G>::value;
+    auto* kernel = total >= cpdp::kOnceMinElements && total <= cpdp::kOnceMaxElements
+                       ? cpdp::local_step_kernel<cpdp::kOptSGD, G, cpdp::kLocalUnroll, warp_runs, true>
+                       : cpdp::local_step_kernel<cpdp::kOptSGD, G, cpdp::kLocalUnroll, warp_runs, false>;
+    return launch(c, kernel, grid, s, c->params, c->mom, static_cast<float*>(nullptr), g, total, a, turn(c));
 }
 
 // The one-pass reconcile for at most Shape::wmax workers.

@@ -98,6 +98,10 @@ struct GradLoad<float> {
     static __device__ __forceinline__ float4 vec4(const float* g, int64_t q) {
         return __ldg(reinterpret_cast<const float4*>(g) + q);
     }
+    // the same, first out of L2 (a gradient is read once)
+    static __device__ __forceinline__ float4 vec4_once(const float* g, int64_t q) {
+        return __ldcs(reinterpret_cast<const float4*>(g) + q);
+    }
     static __device__ __forceinline__ float one(const float* g, int64_t e) { return __ldg(g + e); }
     // the group's raw words, widened only when summed (identical for float32)
     using Words = float4;
@@ -113,9 +117,10 @@ struct GradLoad<float> {
 template <>
 struct GradLoad<bf16_bits> {
     static __device__ __forceinline__ float4 vec4(const bf16_bits* g, int64_t q) {
-        const uint2 u = __ldg(reinterpret_cast<const uint2*>(g) + q);
-        return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
-                           __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+        return widen(__ldg(reinterpret_cast<const uint2*>(g) + q));
+    }
+    static __device__ __forceinline__ float4 vec4_once(const bf16_bits* g, int64_t q) {
+        return widen(__ldcs(reinterpret_cast<const uint2*>(g) + q));
     }
     static __device__ __forceinline__ float one(const bf16_bits* g, int64_t e) {
         return bf16_widen(__ldg(reinterpret_cast<const unsigned short*>(g) + e));
@@ -309,8 +314,7 @@ __device__ __forceinline__ void pdl_wait_then_release() {
 // alternating: LocalSGD N = 2^22, W = 4 191 -> 172; CPDP N = 8 M, W = 2, K = 8
 // 389 -> 338; N = 2^20, W = 8 91.6 -> 85.3; AdamW N = 2^24, W = 1 312 -> 287;
 // N = 2^21, W = 8 281 -> 260; ResNet-50 W = 8 2,165 -> 2,151 (what stays in L2
-// is then 2 % of the state). Evict-first gradient loads on top, to leave the
-// state more of L2, measured 1 to 8 % slower at most sizes (ResNet-50 2,324).
+// is then 2 % of the state).
 __device__ __forceinline__ unsigned walk_block(int backwards) {
     return backwards ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
 }
@@ -378,8 +382,9 @@ struct LocalStepBlocks {
 
 // WARP_RUNS picks which U vectors a thread takes: with it, each warp streams
 // U * 512 contiguous bytes of every array (vectors 32 apart); without it, the
-// block's 256 threads cover 4 KB and a thread's vectors are 4 KB apart.
-template <int OPT, typename G, int U, bool WARP_RUNS>
+// block's 256 threads cover 4 KB and a thread's vectors are 4 KB apart. ONCE
+// loads the gradients evict-first, which leaves more of L2 to the state.
+template <int OPT, typename G, int U, bool WARP_RUNS, bool ONCE>
 __global__ void __launch_bounds__(kThreads, LocalStepBlocks<OPT>::value)
 local_step_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
                   const G* __restrict__ grads, int64_t total, StepArgs a, int backwards) {
@@ -400,7 +405,7 @@ local_step_kernel(float* __restrict__ params, float* __restrict__ mom, float* __
                 th[u] = p4[CPDP_IDX(q, nq)];
                 bu[u] = m4[CPDP_IDX(q, nq)];
                 if (OPT == kOptAdamW) sv[u] = s4[CPDP_IDX(q, nq)];
-                gr[u] = GradLoad<G>::vec4(grads, CPDP_IDX(q, nq));
+                gr[u] = ONCE ? GradLoad<G>::vec4_once(grads, CPDP_IDX(q, nq)) : GradLoad<G>::vec4(grads, CPDP_IDX(q, nq));
             }
         }
 #pragma unroll
