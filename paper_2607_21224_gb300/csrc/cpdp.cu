@@ -260,29 +260,34 @@ template <typename Shape, int METHOD, int OPT, bool SS, typename G>
 cudaError_t launch_onepass(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, const cpdp::SyncArgs& a, int64_t nq) {
     static_assert(Shape::use, "a one-pass shape that is not used");
     c->reconcile_kernel = "reconcile_onepass_kernel";
-    return launch(c, cpdp::reconcile_onepass_kernel<METHOD, OPT, SS, G, Shape::wmax, Shape::min_blocks>,
-                  cpdp::grid_for(nq, cpdp::kThreads), s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
+    const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N);
+    return cpdp::launch_shaped(
+        c->pdl, cpdp::reconcile_onepass_kernel<METHOD, OPT, SS, G, Shape::wmax, Shape::min_blocks>,
+        cpdp::grid_for(nq, threads), threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
 }
 
 // The vectorised reconcile in launch shape Shape, with 32-bit offsets where
 // the shape asks for them and the sizes allow.
 template <typename Shape, int METHOD, int OPT, bool SS, typename G>
 cudaError_t launch_vec4(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, const cpdp::SyncArgs& a, int64_t nq) {
-    const unsigned grid = cpdp::grid_for(nq, cpdp::kThreads);
+    const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N);
+    const unsigned grid = cpdp::grid_for(nq, threads);
     c->reconcile_kernel = "reconcile_vec4_kernel";
     constexpr int grad_rows = cpdp::GradChunkOf<Shape>::rows;
     constexpr bool overlap = cpdp::GradChunkOf<Shape>::overlap;
     if constexpr (Shape::narrow) {
-        if (static_cast<int64_t>(c->W) * nq + static_cast<int64_t>(grid) * cpdp::kThreads < (int64_t(1) << 31))
-            return launch(c,
-                          cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks, Shape::late,
-                                                      int32_t, grad_rows, overlap>,
-                          grid, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, static_cast<int32_t>(nq), a, turn(c));
+        if (static_cast<int64_t>(c->W) * nq + static_cast<int64_t>(grid) * threads < (int64_t(1) << 31))
+            return cpdp::launch_shaped(
+                c->pdl,
+                cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks, Shape::late, int32_t,
+                                            grad_rows, overlap>,
+                grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, static_cast<int32_t>(nq), a,
+                turn(c));
     }
-    return launch(c,
-                  cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks, Shape::late, int64_t,
-                                              grad_rows, overlap>,
-                  grid, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
+    return cpdp::launch_shaped(c->pdl,
+                               cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks,
+                                                           Shape::late, int64_t, grad_rows, overlap>,
+                               grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
 }
 
 template <int METHOD, int OPT, bool SS, typename G>

@@ -15,11 +15,12 @@ namespace {
 template <typename Shape, int METHOD, int OPT, bool SS, typename G, int V, int U, typename Idx>
 cudaError_t launch_shape(const ReconcileCall& c) {
     const int64_t units = c.N / V;
-    const unsigned grid = grid_for((units + 32 * U - 1) / (32 * U), kThreads / 32);
+    const int threads = reconcile_threads(METHOD, OPT, SS, c.W, c.N);
+    const unsigned grid = grid_for((units + 32 * U - 1) / (32 * U), threads / 32);
     return launch_shaped(c.pdl,
                          reconcile_scalar_kernel<METHOD, OPT, SS, G, V, U, Shape::rows, Shape::min_blocks, Shape::late, Idx,
                                                  Shape::grad_rows, Shape::overlap && METHOD != kMethodLocalSGD>,
-                         grid, kThreads, 0, c.stream, c.params, c.mom, c.sq, static_cast<const G*>(c.grads), c.anchor,
+                         grid, threads, 0, c.stream, c.params, c.mom, c.sq, static_cast<const G*>(c.grads), c.anchor,
                          c.slow_v, c.W, static_cast<Idx>(units), c.args, c.backwards);
 }
 

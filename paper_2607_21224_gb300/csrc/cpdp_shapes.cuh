@@ -43,6 +43,24 @@ inline unsigned grid_for(int64_t work_items, int64_t per_block) {
     return static_cast<unsigned>(blocks);
 }
 
+// Threads per block of a reconcile's column kernels (they are compiled for up
+// to kThreads, and for the registers of that many). An SM holds the same warps
+// either way, but with few blocks a small one leaves fewer SMs with one block
+// more than the others, and its barrier-free warps retire one by one: 64
+// threads against 256, time ratio, at N = 20,000 to 320,000 1.00-1.15 (W = 8,
+// N = 60,000 3.9 -> 3.4 us), 700,000 1.00-1.10, 1 to 3 million 1.00-1.05. Above
+// 4 million columns the two are within 0.4 % (64 slower), except where they
+// favour 64: state-reconciling AdamW (ViT-S, W = 8 1.010, W = 32 1.027) and CPDP
+// at odd N (W = 4, 23.7 M: bf16 SGD 1.014, AdamW 1.012). One worker's blocks are
+// so short that the rate at which the GPU starts blocks, about one per ns,
+// bounds 64-thread ones (N = 2^26, DDP SGD: 170 -> 264 us).
+constexpr int kThreadsSmall = 64;
+inline int reconcile_threads(int method, int opt, bool state_sync, int W, int64_t N) {
+    if (W == 1) return N <= (int64_t(1) << 20) ? kThreadsSmall : kThreads;
+    const bool always = (opt == kOptAdamW && state_sync) || (method == kMethodCPDP && (N & 1) != 0);
+    return always || N <= (int64_t(1) << 22) ? kThreadsSmall : kThreads;
+}
+
 // Rows per load chunk of the vectorised reconcile, the resident blocks per SM it
 // is compiled for (3 blocks of 256 threads: 80 registers; 4 blocks: 64),
 // whether theta_ref and v are loaded after the rows (late) to free registers,
