@@ -2,7 +2,8 @@
 //
 // Host side only: argument validation, the context, the synchronization
 // schedule (eq. 4 with the epoch-end rule of Sec. 3.1) and kernel launches.
-// Every step of the path itself runs in the kernels of cpdp_kernels.cuh.
+// Every step of the path itself runs in the kernels of cpdp_kernels.cuh (and
+// cpdp_split.cuh, cpdp_tma.cuh, cpdp_shuffle.cuh).
 #include "cpdp.h"
 #include "cpdp_floor.cuh"
 #include "cpdp_kernels.cuh"

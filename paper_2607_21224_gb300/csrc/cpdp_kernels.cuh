@@ -7,14 +7,17 @@
 // nothing here is a dense contraction.
 //
 // Access pattern: one thread owns a group of 4 consecutive parameters (one
-// 128-bit vector per row). A warp therefore reads or writes 512 contiguous
+// 128-bit vector per row; where N is not a multiple of 4, pairs or single ones
+// a warp apart). A warp therefore reads or writes 512 contiguous
 // bytes of each row it touches; the W-way "strided" reads of the reconcile are
 // W such coalesced segments, one per row, and the W-way sums stay in the
-// thread's registers (no shared memory, no shuffles). Gradients are read
-// through the read-only path; state is read and written with plain
-// write-back accesses. Evict-first (streaming) hints measured slower here: the
-// reconcile lost 6 % with them, because dirty lines pushed out of L2 early
-// reach DRAM as scattered writes instead of combining per DRAM page.
+// thread's registers (no shared memory, no shuffles; many workers over few
+// columns split the rows across warps instead, cpdp_split.cuh). Gradients are
+// read through the read-only path (evict-first in the local step at some
+// sizes); state is read and written with plain
+// write-back accesses. Evict-first (streaming) hints on the state measured
+// slower: the reconcile lost 6 % with them, because dirty lines pushed out of
+// L2 early reach DRAM as scattered writes instead of combining per DRAM page.
 #pragma once
 
 #include <cstdint>

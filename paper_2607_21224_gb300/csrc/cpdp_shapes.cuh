@@ -264,7 +264,7 @@ struct RaggedShape {
     static constexpr bool late = true;
 };
 
-// Few columns: at 4 columns per thread N = 300,000 gives an SM two of the four
+// Few columns: at 4 columns per thread N = 300,000 gives an SM two of the four 256-thread
 // blocks it can hold, so up to kRaggedNarrowColumns a thread owns one load's
 // columns instead and 4-row chunks keep it busy (W = 8, N = 100,001, us, one
 // column and one row at a time / 4 columns / this: CPDP SGD f32 5.15 / 5.87 /
