@@ -59,6 +59,20 @@ inline int split_warps(int W, int64_t tiles) {
     return warps;
 }
 
+// Whether a warp has rows enough for deeper chunks than 4 rows: 8 gradient rows
+// for float32 pairs (SGD), 8 gradient and 8 state rows at odd N, where a row is
+// one register. Sync step, us, 4-row chunks -> these: CPDP SGD f32 W = 64,
+// N = 60,000 15.6 -> 14.9, N = 60,001 23.1 -> 16.2; W = 200, N = 13,215 21.7 ->
+// 16.3; state-reconciling SGD f32 W = 64, N = 120,000 32.3 -> 28.3; DDP SGD f32
+// W = 64, N = 60,001 18.9 -> 15.4; AdamW bf16 W = 200, N = 60,001 75.1 -> 72.3. With
+// fewer rows per warp the deeper chunks are mostly empty and 5 to 20 % slower
+// (W = 16, N = 20,001 2.8 -> 3.4; 16 warps, W = 64, N = 5,001 3.6 -> 4.0), as is
+// state-reconciling SGD at 8 warps and odd N (W = 64, N = 13,215 6.3 -> 7.0).
+constexpr int64_t kSplitManyTiles = 1000;
+inline bool split_deep(int W, int warps, int64_t tiles) {
+    return warps <= 8 && (W >= 64 || (W >= 24 && tiles >= kSplitManyTiles));
+}
+
 // V consecutive columns of one row.
 template <int V>
 struct Slice {

@@ -48,7 +48,9 @@ def test_split_rows_match_the_column_kernels(N, W):
 @pytest.mark.parametrize("W,N,want", [
     (8, 1200, "reconcile_vec4_kernel"), (9, 64_000, "reconcile_split_kernel"), (9, 64_004, "reconcile_vec4_kernel"),
     (16, 160_000, "reconcile_split_kernel"), (23, 24_001, None), (24, 63_999, "reconcile_split_kernel"),
-    (24, 64_001, None), (9, 159_999, None), (4096, 66, "reconcile_split_kernel")])
+    (24, 64_001, None), (9, 159_999, None), (24, 31_999, "reconcile_split_kernel"), (24, 32_001, "reconcile_split_kernel"),
+    (24, 64_002, "reconcile_split_kernel"), (63, 8_194, "reconcile_split_kernel"), (65, 8_195, "reconcile_split_kernel"),
+    (100, 60_001, "reconcile_split_kernel"), (4096, 66, "reconcile_split_kernel")])
 def test_the_rule_that_selects_it(W, N, want):
     if W * WIDE > 1 << 26:  # 4,096 workers: a wider problem of its own size
         gen = torch.Generator(device="cuda").manual_seed(1)
