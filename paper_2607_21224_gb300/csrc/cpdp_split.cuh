@@ -34,18 +34,34 @@ constexpr int kSplitMaxWarps = 16;
 // 200,000 1.04-1.27, 400,000 0.92-1.02. Odd N, W = 9: 20,001 1.24-1.32,
 // 60,001 0.79-0.85; W = 24: 60,001 1.11-1.25, 100,001 0.87-1.02; W = 64:
 // 60,001 1.27-1.44, 100,001 1.01-1.15.
-// Odd rows cost the column kernels more with float32 gradients and no velocity
-// to update: DDP SGD f32 1.05-1.94 up to N = 300,001 at any W from 9 (W = 64, N = 100,001 39.2 ->
-// 28.6 us); LocalSGD and AdamW f32 from 16 workers 1.02-1.20 at 100,001 and 0.88-1.04 at
-// 150,001.
+// Odd rows cost the column kernels more where a row is more of 4-byte loads,
+// and this kernel holds 8 of them at once (split_deep), so its range is longer
+// at odd N: float32 gradients, SGD from 24 workers to 300,001 1.05-1.60 for
+// CPDP, 1.03-1.29 for LocalSGD, and for DDP from 9 workers 1.05-2.0; AdamW from
+// 24 workers to 420,001 1.01-1.55 for DDP and LocalSGD, for CPDP to 100,001
+// 1.03-1.22 (0.86-1.08 to 300,001) and from 100 workers to 300,001 1.0-1.26;
+// bf16 from 48 workers to 100,001 1.03-1.19 (0.89-1.05 at 150,001). State
+// reconciliation from 100 workers to 300,001, AdamW and LocalSGD: 1.02-1.45;
+// CPDP SGD 0.90-1.14, so it keeps 64,000.
 inline bool split_takes(const ReconcileCall& c) {
     if (c.W < 9) return false;
     if ((c.N & 1) == 0) return c.N <= (c.W < 16 ? 64'000 : 160'000);
-    if (!c.bf16 && !c.state_sync) {
-        if (c.method == kMethodDDP && c.opt == kOptSGD) return c.N <= 300'000;
-        if ((c.method != kMethodCPDP || c.opt == kOptAdamW) && c.W >= 16) return c.N <= 110'000;
+    const bool sgd = c.opt == kOptSGD, cpdp_method = c.method == kMethodCPDP;
+    int64_t limit = c.W < 24 ? 24'000 : 64'000;
+    if (c.state_sync) {
+        if (c.W >= 100 && (!sgd || !cpdp_method)) limit = 300'000;
+    } else if (c.bf16) {
+        if (c.W >= 48) limit = 110'000;
+    } else if (sgd && (c.method == kMethodDDP || c.W >= 24)) {
+        limit = 300'000;
+    } else if (!sgd && c.W >= 24 && !cpdp_method) {
+        limit = 420'000;
+    } else if (!sgd && c.W >= 100) {
+        limit = 300'000;
+    } else if (c.W >= 16 && (!sgd || !cpdp_method)) {
+        limit = 110'000;
     }
-    return c.N <= (c.W < 24 ? 24'000 : 64'000);
+    return c.N <= limit;
 }
 
 // Warps per block over `tiles` blocks: more while the launch stays within
