@@ -261,7 +261,7 @@ template <typename Shape, int METHOD, int OPT, bool SS, typename G>
 cudaError_t launch_onepass(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, const cpdp::SyncArgs& a, int64_t nq) {
     static_assert(Shape::use, "a one-pass shape that is not used");
     c->reconcile_kernel = "reconcile_onepass_kernel";
-    const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N);
+    const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N, 4);
     return cpdp::launch_shaped(
         c->pdl, cpdp::reconcile_onepass_kernel<METHOD, OPT, SS, G, Shape::wmax, Shape::min_blocks>,
         cpdp::grid_for(nq, threads), threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
@@ -271,7 +271,7 @@ cudaError_t launch_onepass(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, c
 // the shape asks for them and the sizes allow.
 template <typename Shape, int METHOD, int OPT, bool SS, typename G>
 cudaError_t launch_vec4(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, const cpdp::SyncArgs& a, int64_t nq) {
-    const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N);
+    const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N, 4);
     const unsigned grid = cpdp::grid_for(nq, threads);
     c->reconcile_kernel = "reconcile_vec4_kernel";
     constexpr int grad_rows = cpdp::GradChunkOf<Shape>::rows;

@@ -15,7 +15,7 @@ namespace {
 template <typename Shape, int METHOD, int OPT, bool SS, typename G, int V, int U, typename Idx>
 cudaError_t launch_shape(const ReconcileCall& c) {
     const int64_t units = c.N / V;
-    const int threads = reconcile_threads(METHOD, OPT, SS, c.W, c.N);
+    const int threads = reconcile_threads(METHOD, OPT, SS, c.W, c.N, U * V);
     const unsigned grid = grid_for((units + 32 * U - 1) / (32 * U), threads / 32);
     return launch_shaped(c.pdl,
                          reconcile_scalar_kernel<METHOD, OPT, SS, G, V, U, Shape::rows, Shape::min_blocks, Shape::late, Idx,
@@ -40,7 +40,7 @@ struct Ragged {
     // one load per thread and row for few columns, kRaggedColumns / 32 columns per thread for more
     template <typename Narrow, typename Wide, int METHOD, int OPT, bool SS, typename G, int V>
     cudaError_t by_size() const {
-        if (c.N <= kRaggedNarrowColumns<V, OPT, SS> && static_cast<int64_t>(c.W) * c.N < (int64_t(1) << 30))
+        if (c.N <= ragged_narrow_columns<V, OPT, SS>(c.W) && static_cast<int64_t>(c.W) * c.N < (int64_t(1) << 30))
             return launch_shape<Narrow, METHOD, OPT, SS, G, V, 1, int32_t>(c);
         constexpr int U = kRaggedColumns / (32 * V);
         // the largest offset formed is below W rows plus one grid-wide step

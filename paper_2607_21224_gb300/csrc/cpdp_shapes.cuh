@@ -51,12 +51,14 @@ inline unsigned grid_for(int64_t work_items, int64_t per_block) {
 // N = 60,000 3.9 -> 3.4 us), 700,000 1.00-1.10, 1 to 3 million 1.00-1.05. Above
 // 4 million columns the two are within 0.4 % (64 slower), except where they
 // favour 64: state-reconciling AdamW (ViT-S, W = 8 1.010, W = 32 1.027) and CPDP
-// at odd N (W = 4, 23.7 M: bf16 SGD 1.014, AdamW 1.012). One worker's blocks are
-// so short that the rate at which the GPU starts blocks, about one per ns,
-// bounds 64-thread ones (N = 2^26, DDP SGD: 170 -> 264 us).
+// at odd N (W = 4, 23.7 M: bf16 SGD 1.014, AdamW 1.012). The GPU starts about
+// one block per ns: where a 64-thread block is shorter than that (few workers,
+// few columns per thread) it bounds the launch (one worker, N = 2^26, DDP SGD:
+// 170 -> 264 us), so such launches take 64 threads only while they are small.
 constexpr int kThreadsSmall = 64;
-inline int reconcile_threads(int method, int opt, bool state_sync, int W, int64_t N) {
-    if (W == 1) return N <= (int64_t(1) << 20) ? kThreadsSmall : kThreads;
+inline int reconcile_threads(int method, int opt, bool state_sync, int W, int64_t N, int columns_per_thread) {
+    if (W * columns_per_thread < 6)
+        return N <= int64_t(1024) * columns_per_thread * kThreadsSmall * columns_per_thread ? kThreadsSmall : kThreads;
     const bool always = (opt == kOptAdamW && state_sync) || (method == kMethodCPDP && (N & 1) != 0);
     return always || N <= (int64_t(1) << 22) ? kThreadsSmall : kThreads;
 }
@@ -265,7 +267,7 @@ struct RaggedShape {
 };
 
 // Few columns: at 4 columns per thread N = 300,000 gives an SM two of the four 256-thread
-// blocks it can hold, so up to kRaggedNarrowColumns a thread owns one load's
+// blocks it can hold, so up to ragged_narrow_columns a thread owns one load's
 // columns instead and 4-row chunks keep it busy (W = 8, N = 100,001, us, one
 // column and one row at a time / 4 columns / this: CPDP SGD f32 5.15 / 5.87 /
 // 4.29; N = 300,002 AdamW bf16 15.1 / 16.2 / 12.7). The lines are where the two
@@ -275,18 +277,28 @@ struct RaggedShape {
 // and 11.8; N = 600,002 18.7 and 17.8; AdamW f32 at N = 600,002 25.0 and 30.9,
 // at 2,000,002 76.5 and 75.5). State-reconciling SGD stores nothing inside its
 // row loop and holds little per column, so 1-row chunks at 8 blocks of single
-// columns are as good as any up to 700,000 odd columns (W = 8, N = 300,001
-// 10.4 us; at 6 blocks 12.0, 4-row chunks 12.4) and beat pairs up to
+// columns are as good as any up to 700,000 odd columns below 24 workers (W = 8,
+// N = 300,001 10.4 us; at 6 blocks 12.0, 4-row chunks 12.4; W = 141, N = 351,435
+// 249, the wide shape 209) and beat pairs up to
 // kRaggedSinglesColumns even ones (W = 4, N = 100,002 2.5 us against 2.8).
+// State-reconciling AdamW is short of registers for the overlapped chunk and
+// takes 5 blocks without it (W = 8, N = 300,001 15.2 and 14.0 us for float32
+// and bf16 gradients, overlapped at 4 blocks 15.9 and 14.5).
 constexpr int64_t kRaggedSinglesColumns = 200'000;
 template <int V, int OPT, bool SS>
-constexpr int64_t kRaggedNarrowColumns = V == 2 ? (OPT == kOptAdamW || SS ? 1'500'000 : 500'000)
-                                                : (OPT == kOptAdamW ? 400'000 : SS ? 700'000 : 250'000);
+inline int64_t ragged_narrow_columns(int W) {
+    if (W == 1) return V == 2 ? 450'000 : 150'000;
+    if (V == 2) return OPT == kOptAdamW || SS ? 1'500'000 : 500'000;
+    if (OPT == kOptAdamW) return 400'000;
+    return SS && W < 24 ? 700'000 : 250'000;
+}
 template <int V, int OPT, bool SS, typename G>
 struct RaggedShapeNarrow {
-    static constexpr bool overlap = !(SS && OPT == kOptSGD);
-    static constexpr int rows = overlap ? 4 : 1, min_blocks = overlap || V == 2 ? 4 : 8;
-    static constexpr int grad_rows = !overlap ? 1 : std::is_same<G, float>::value ? 4 : 8;
+    static constexpr bool one_row = SS && OPT == kOptSGD, plain_chunks = V == 1 && SS && OPT == kOptAdamW;
+    static constexpr bool overlap = !one_row && !plain_chunks;
+    static constexpr int rows = one_row ? 1 : 4;
+    static constexpr int min_blocks = plain_chunks ? 5 : V == 1 && one_row ? 8 : 4;
+    static constexpr int grad_rows = one_row ? 1 : std::is_same<G, float>::value ? 4 : 8;
     static constexpr bool late = true;
 };
 
