@@ -4,16 +4,17 @@
 // What bounds the column kernels there: one thread walks all W rows of its
 // columns, a chunk at a time, so a launch takes about W / 2 dependent trips to
 // memory however few columns there are, and N / 1024 blocks cannot fill 152
-// SMs (W = 64, N = 60,000: 59 blocks, 32.8 us for 78 MB). Here a block owns 32 loads' columns
-// (64 at even N, 32 at odd) and its 4 to 16 warps take every R-th row, so a
-// column's rows are loaded by R warps at once and N / 64 blocks run. The
-// values to be averaged pass through shared memory, where one thread per
-// column adds them in worker order: the sums are those of the other kernels
-// bit for bit (partial sums per warp measured the same within 10 %, but in
-// another order). Sync step, us, column kernels -> this one, CPDP SGD f32: W = 64,
-// N = 60,000 32.8 -> 15.6 (5.0 TB/s; the bytes take 11.4 at the copy rate);
-// W = 16, N = 20,000 5.54 -> 2.26; W = 200, N = 20,000 90.6 -> 22.9; AdamW bf16
-// W = 64, N = 20,000 4.5 times as fast.
+// SMs (W = 64, N = 60,000: 59 blocks, 32.8 us for 78 MB). Here a block owns the
+// columns of 32 loads (64 at even N, 32 at odd) and its 4 to 16 warps take
+// every R-th row, so a column's rows are loaded by R warps at once and N / 64
+// (N / 32) blocks run. The values to be averaged pass through shared memory,
+// where one thread per column adds them in worker order: the sums are those of
+// the other kernels bit for bit (partial sums per warp measured the same
+// within 10 %, but in another order). Sync step, us, column kernels -> this one,
+// CPDP SGD f32: W = 64, N = 60,000 32.8 -> 14.9 (5.2 TB/s; the bytes take 11.4
+// at the copy rate); W = 16, N = 20,000 5.54 -> 2.26; W = 200, N = 20,000 90.6 ->
+// 22.2; AdamW bf16 W = 64, N = 20,000 47 -> 10.4. What bounds it now is the trips
+// that are left, two to six per 64 rows, and the barriers between them.
 #pragma once
 
 #include <cstdint>
@@ -31,13 +32,12 @@ constexpr int kSplitMaxWarps = 16;
 // their longer row segments win (ratio of sync-step times, column kernel over
 // this one): even N, W = 9: N = 60,000 1.17-1.40 for SGD, 100,000 0.85-1.18;
 // W = 16: 100,000 1.04-1.61, 200,000 0.85-1.24; W = 64: 100,000 1.26-1.72,
-// 200,000 1.04-1.27, 400,000 0.92-1.02. Odd N, W = 9: 20,001 1.24-1.32,
-// 60,001 0.79-0.85; W = 24: 60,001 1.11-1.25, 100,001 0.87-1.02; W = 64:
-// 60,001 1.27-1.44, 100,001 1.01-1.15.
-// Odd rows cost the column kernels more where a row is more of 4-byte loads,
-// and this kernel holds 8 of them at once (split_deep), so its range is longer
+// 200,000 1.04-1.27, 400,000 0.92-1.02. Odd N: W = 9 20,001 1.24-1.32, 60,001
+// 0.79-0.85; W = 24 and more 64,003 1.00-2.0.
+// Odd rows cost the column kernels more, as a row is more of 4-byte loads, and
+// this kernel holds 8 of them at once (split_deep), so its range is longer
 // at odd N: float32 gradients, SGD from 24 workers to 300,001 1.05-1.60 for
-// CPDP, 1.03-1.29 for LocalSGD, and for DDP from 9 workers 1.05-2.0; AdamW from
+// CPDP, 1.03-1.29 for LocalSGD, and for DDP from 9 workers 0.96-2.0; AdamW from
 // 24 workers to 420,001 1.01-1.55 for DDP and LocalSGD, for CPDP to 100,001
 // 1.03-1.22 (0.86-1.08 to 300,001) and from 100 workers to 300,001 1.0-1.26;
 // bf16 from 48 workers to 100,001 1.03-1.19 (0.89-1.05 at 150,001). State
