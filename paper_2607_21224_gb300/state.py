@@ -11,6 +11,11 @@ import torch
 
 from . import cpdp as _c
 
+# The current stream's handle without a Stream object around it: 0.1 us instead
+# of 3.4. The function is private to torch, so a torch without it is served by
+# the public one.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
 
 def grad_dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.float32:
@@ -48,8 +53,9 @@ class CPDPState:
     # A small step's cost is these calls: the kernels take 2 us, the launch 2 us.
     def _stream(self, stream) -> int:
         if stream is None:
-            # the current stream's handle without a Stream object around it: 0.1 us instead of 3.4
-            return torch._C._cuda_getCurrentRawStream(self._device_index)
+            if _raw_stream is not None:
+                return _raw_stream(self._device_index)
+            stream = torch.cuda.current_stream(self._device_index)
         return stream if isinstance(stream, int) else stream.cuda_stream
 
     def _grads(self, grads: torch.Tensor) -> torch.Tensor:
