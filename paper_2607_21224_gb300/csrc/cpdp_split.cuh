@@ -43,8 +43,10 @@ constexpr int kSplitMaxWarps = 16;
 // bf16 from 48 workers to 100,001 1.03-1.19 (0.89-1.05 at 150,001). State
 // reconciliation from 100 workers to 300,001, AdamW and LocalSGD: 1.02-1.45;
 // CPDP SGD 0.90-1.14, so it keeps 64,000.
+// Its offsets are 32-bit: W rows of N / V loads stay below 2^31.
 inline bool split_takes(const ReconcileCall& c) {
-    if (c.W < 9) return false;
+    const int64_t units = (c.N & 1) == 0 ? c.N >> 1 : c.N;
+    if (c.W < 9 || c.W * units >= int64_t(1) << 31) return false;
     if ((c.N & 1) == 0) return c.N <= (c.W < 16 ? 64'000 : 160'000);
     const bool sgd = c.opt == kOptSGD, cpdp_method = c.method == kMethodCPDP;
     int64_t limit = c.W < 24 ? 24'000 : 64'000;
