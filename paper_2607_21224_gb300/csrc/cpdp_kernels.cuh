@@ -391,6 +391,7 @@ template <int OPT, typename G, int U, bool WARP_RUNS, bool ONCE>
 __global__ void __launch_bounds__(kThreads, LocalStepBlocks<OPT>::value)
 local_step_kernel(float* __restrict__ params, float* __restrict__ mom, float* __restrict__ sq,
                   const G* __restrict__ grads, int64_t total, StepArgs a, int backwards) {
+    const unsigned block = walk_block(backwards);
     pdl_wait_then_release();
     const int64_t nq = total >> 2;
     float4* p4 = reinterpret_cast<float4*>(params);
@@ -399,7 +400,7 @@ local_step_kernel(float* __restrict__ params, float* __restrict__ mom, float* __
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * U;
     const int64_t first = WARP_RUNS ? (int64_t)(threadIdx.x / 32) * 32 * U + threadIdx.x % 32 : threadIdx.x;
     const int64_t step = WARP_RUNS ? 32 : blockDim.x;
-    for (int64_t q0 = (int64_t)walk_block(backwards) * blockDim.x * U + first; q0 < nq; q0 += stride) {
+    for (int64_t q0 = (int64_t)block * blockDim.x * U + first; q0 < nq; q0 += stride) {
         float4 th[U], bu[U], sv[U], gr[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
