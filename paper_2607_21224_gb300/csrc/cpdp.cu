@@ -235,8 +235,11 @@ cpdp_status check_grads(cpdp_ctx* ctx, const void* grads, cpdp_dtype dtype) {
     return CPDP_OK;
 }
 
-// The walk direction of the launch being made; the next one goes the other way.
-int turn(cpdp_ctx* c) { return c->backwards ^= 1; }
+// The walk direction of the launch being made: where launches alternate, the
+// next one goes the other way.
+int turn(cpdp_ctx* c) {
+    return cpdp::walks_alternate(c->W, c->N, c->optimizer == CPDP_OPT_ADAMW) ? c->backwards ^= 1 : 0;
+}
 
 template <typename G>
 cudaError_t launch_local(cpdp_ctx* c, const void* grads, cudaStream_t s, const cpdp::StepArgs& a) {

@@ -310,10 +310,11 @@ __device__ __forceinline__ void pdl_wait_then_release() {
 // The block's place in the walk over the arrays. A launch leaves the part of
 // the state that it touched last in L2, dirty; a next launch that starts at
 // the other end has evicted it before it gets there. So launches of one
-// context alternate between walking forwards and backwards: each starts on
-// what the one before left, and those lines are read and written again without
-// going to DRAM. Which columns a block takes is all that changes, so the bits
-// do not. K-period at K = 4 and float32 SGD unless stated, us, one direction ->
+// context alternate between walking forwards and backwards where the state is
+// too large for L2 to keep (walks_alternate): each starts on what the one
+// before left, and those lines are read and written again without going to
+// DRAM. Which columns a block takes is all that changes, so the bits do not.
+// K-period at K = 4 and float32 SGD unless stated, us, one direction ->
 // alternating: LocalSGD N = 2^22, W = 4 191 -> 172; CPDP N = 8 M, W = 2, K = 8
 // 389 -> 338; N = 2^20, W = 8 91.6 -> 85.3; AdamW N = 2^24, W = 1 312 -> 287;
 // N = 2^21, W = 8 281 -> 260; ResNet-50 W = 8 2,165 -> 2,151 (what stays in L2

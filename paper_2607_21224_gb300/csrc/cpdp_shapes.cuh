@@ -32,6 +32,20 @@ struct LocalWarpRuns {
 // 0.97-1.04. AdamW gains 0.6 % at best; the reconcile, which reads fewer
 // gradients per state byte, 1 % at best.
 constexpr int64_t kOnceMinElements = 6'000'000, kOnceMaxElements = int64_t(1) << 25;
+
+// Whether a context's launches alternate their walk direction (walk_block):
+// where the replicas and optimizer states (about half of L2 and more) no longer
+// stay in L2 from one launch to the next. Below that there is nothing to gain,
+// and a run of sync steps loses, as a block's columns move to another SM, and
+// mostly to the other die, each time. Back-to-back sync steps on one state, N a
+// multiple of 4, one direction over alternating, geometric means over the
+// variants: 1 to 3 MB 0.95-0.97, 5 to 13 MB 0.97-0.98, 20 to 50 MB 0.99-1.00, 56 MB
+// 0.97, 64 MB 1.02, 70 MB 1.05, 80 MB 1.07, 87 to 110 MB 1.12-1.21, 170 MB 1.12.
+// Periods of 2 and 4 steps: 0.996-1.01 to 49 MB, 61 MB 1.014, 75 MB 1.07, 93 MB 1.13.
+constexpr int64_t kAlternateMinStateBytes = 60'000'000;
+inline bool walks_alternate(int64_t W, int64_t N, bool adamw) {
+    return W * N * (adamw ? 12 : 8) >= kAlternateMinStateBytes;
+}
 constexpr int64_t kMaxGrid = 0x7fffffff;
 
 // Blocks for `work_items` items at `per_block` items per block (kernels loop

@@ -1,0 +1,67 @@
+"""The rules that choose a launch (host functions of the kernel headers),
+compiled into a small program and run on the CPU."""
+import subprocess
+
+import pytest
+
+from paper_2607_21224_gb300 import build
+
+CODES = {"cpdp": 0, "localsgd": 1, "ddp": 2}
+VARIANTS = [(m, o, s, b) for m in CODES for o in ("sgd", "adamw") for s in (False, True) for b in (False, True)
+            if not (m == "ddp" and s)]
+
+PROGRAM = r"""
+#include "cpdp_shapes.cuh"
+#include "cpdp_split.cuh"
+#include <cstdio>
+int main() {
+    cpdp::ReconcileCall c{};
+    int method, opt, state_sync, bf16, W;
+    long long N;
+    while (std::scanf("%d %d %d %d %d %lld", &method, &opt, &state_sync, &bf16, &W, &N) == 6) {
+        c.method = method, c.opt = opt, c.state_sync = state_sync != 0, c.bf16 = bf16 != 0, c.W = W, c.N = N;
+        std::printf("%d %d", cpdp::split_takes(c) ? 1 : 0, cpdp::walks_alternate(W, N, opt == cpdp::kOptAdamW) ? 1 : 0);
+        std::printf("\n");
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    """rules(calls) for each call (method, opt, state_sync, bf16, W, N): taken by the split kernel; walk direction
+    alternates."""
+    folder = tmp_path_factory.mktemp("launch_rules")
+    source, program = folder / "rules.cu", folder / "rules"
+    source.write_text(PROGRAM)
+    subprocess.run([build.nvcc_path(), "-std=c++17", *build.ARCH, f"-I{build.INCLUDE}", f"-I{build.CSRC}", "-o",
+                    str(program), str(source)], check=True, capture_output=True, text=True)
+
+    def run(calls):
+        lines = "".join(f"{CODES[m]} {int(o == 'adamw')} {int(s)} {int(b)} {W} {N}\n" for m, o, s, b, W, N in calls)
+        r = subprocess.run([str(program)], input=lines, capture_output=True, text=True, check=True)
+        return [tuple(map(int, line.split())) for line in r.stdout.splitlines()]
+    return run
+
+
+def test_no_split_call_passes_32_bit_offsets(rules):
+    """The kernel's offsets are 32-bit: W rows of N / V loads must stay below 2^31, whatever the limits on W and N."""
+    calls = [(*v, W, N) for v in VARIANTS for W in (9, 64, 1000, 4096, 8192, 1 << 15, 1 << 20, 1 << 24, 1 << 28)
+             for N in (2, 3, 1_001, 4_096, 60_001, 160_000, 300_001, 419_999, 420_000)]
+    taken = [split for split, *_ in rules(calls)]
+    assert any(taken)
+    for (*v, W, N), got in zip(calls, taken):
+        if got:
+            assert W * (N // (2 if N % 2 == 0 else 1)) < 1 << 31, (*v, W, N)
+
+
+def test_walks_alternate_only_past_what_l2_keeps(rules):
+    """Below half of L2 the state is there anyway, and a block that moves to another SM each time loses by it."""
+    sizes = [(1, 7_499_999, 4_999_999), (4, 1_874_999, 1_249_999), (8, 937_499, 624_999), (60, 124_999, 83_333)]
+    below = [("cpdp", o, False, False, W, n) for W, sgd, adamw in sizes for o, n in (("sgd", sgd), ("adamw", adamw))]
+    above = [(m, o, s, b, W, n + 1) for m, o, s, b, W, n in below]
+    small = [("cpdp", "sgd", False, False, 4, 3201), ("cpdp", "sgd", False, False, 2, 1 << 20)]
+    large = [("cpdp", "sgd", False, False, 8, 23_712_932), ("localsgd", "sgd", False, False, 4, 1 << 22),
+             ("ddp", "adamw", False, True, 4096, 1 << 28)]
+    assert not any(alternates for _, alternates, *_ in rules(below + small))
+    assert all(alternates for _, alternates, *_ in rules(above + large))
