@@ -65,16 +65,25 @@ inline unsigned grid_for(int64_t work_items, int64_t per_block) {
 // N = 60,000 3.9 -> 3.4 us), 700,000 1.00-1.10, 1 to 3 million 1.00-1.05. Above
 // 4 million columns the two are within 0.4 % (64 slower), except where they
 // favour 64: state-reconciling AdamW (ViT-S, W = 8 1.010, W = 32 1.027) and CPDP
-// at odd N (W = 4, 23.7 M: bf16 SGD 1.014, AdamW 1.012). The GPU starts about
-// one block per ns: where a 64-thread block is shorter than that (few workers,
-// few columns per thread) it bounds the launch (one worker, N = 2^26, DDP SGD:
-// 170 -> 264 us), so such launches take 64 threads only while they are small.
+// at odd N (W = 4, 23.7 M: bf16 SGD 1.014, AdamW 1.012).
+// The GPU starts about one block per ns, and a block shorter than that bounds
+// the launch, so past kThreadsSmallColumns a block gets at least
+// kBlockElements elements of each array (rows times columns: 9 to 25 KB in
+// all). State in L2, sync step, time ratio to 256 threads, geometric means
+// (and the worst) over the variants: W = 1, 4 columns per thread, N = 790,000
+// 64 threads 0.90 (0.70), 1.8 M 0.72 (0.53); W = 2, 1.8 M 0.96 (0.76), 128
+// threads 1.02 (0.98); W = 3 64 threads 1.02-1.05 from 490,000 on. One worker
+// at N = 2^26, DDP SGD: 170 us, with 64 threads 264.
 constexpr int kThreadsSmall = 64;
+constexpr int64_t kThreadsSmallColumns = 65'536;
+constexpr int kBlockElements = 768;
 inline int reconcile_threads(int method, int opt, bool state_sync, int W, int64_t N, int columns_per_thread) {
-    if (W * columns_per_thread < 6)
-        return N <= int64_t(1024) * columns_per_thread * kThreadsSmall * columns_per_thread ? kThreadsSmall : kThreads;
     const bool always = (opt == kOptAdamW && state_sync) || (method == kMethodCPDP && (N & 1) != 0);
-    return always || N <= (int64_t(1) << 22) ? kThreadsSmall : kThreads;
+    if (!always && N > int64_t(1) << 22) return kThreads;
+    int threads = kThreadsSmall;
+    if (N > kThreadsSmallColumns)
+        while (threads < kThreads && int64_t(threads) * columns_per_thread * W < kBlockElements) threads *= 2;
+    return threads;
 }
 
 // Rows per load chunk of the vectorised reconcile, the resident blocks per SM it

@@ -21,6 +21,7 @@ int main() {
     while (std::scanf("%d %d %d %d %d %lld", &method, &opt, &state_sync, &bf16, &W, &N) == 6) {
         c.method = method, c.opt = opt, c.state_sync = state_sync != 0, c.bf16 = bf16 != 0, c.W = W, c.N = N;
         std::printf("%d %d", cpdp::split_takes(c) ? 1 : 0, cpdp::walks_alternate(W, N, opt == cpdp::kOptAdamW) ? 1 : 0);
+        for (int columns : {1, 2, 4}) std::printf(" %d", cpdp::reconcile_threads(method, opt, state_sync, W, N, columns));
         std::printf("\n");
     }
 }
@@ -30,7 +31,7 @@ int main() {
 @pytest.fixture(scope="module")
 def rules(tmp_path_factory):
     """rules(calls) for each call (method, opt, state_sync, bf16, W, N): taken by the split kernel; walk direction
-    alternates."""
+    alternates; threads per block at 1, 2 and 4 columns per thread."""
     folder = tmp_path_factory.mktemp("launch_rules")
     source, program = folder / "rules.cu", folder / "rules"
     source.write_text(PROGRAM)
@@ -65,3 +66,19 @@ def test_walks_alternate_only_past_what_l2_keeps(rules):
              ("ddp", "adamw", False, True, 4096, 1 << 28)]
     assert not any(alternates for _, alternates, *_ in rules(below + small))
     assert all(alternates for _, alternates, *_ in rules(above + large))
+
+
+def test_blocks_last_longer_than_the_gpu_takes_to_start_them(rules):
+    """Past 65,536 columns a block has 768 elements of each array or the most threads there are; above 4 million
+    columns 256 threads, except where smaller blocks gain."""
+    sizes = [65_537, 100_000, 855_424, 1 << 20, 1_800_000, 1 << 22]
+    calls = [(*v, W, N) for v in VARIANTS for W in (1, 2, 3, 4, 5, 6, 8, 64) for N in sizes]
+    for (*v, W, N), (_, _, *threads) in zip(calls, rules(calls)):
+        for columns, t in zip((1, 2, 4), threads):
+            assert t in (64, 128, 256) and (t == 256 or t * columns * W >= 768), (*v, W, N, columns, t)
+            assert t == 64 or t // 2 * columns * W < 768, (*v, W, N, columns, t)
+    small = rules([(*v, W, N) for v in VARIANTS for W in (1, 2, 64) for N in (1, 3201, 65_536)])
+    assert all(t == 64 for _, _, *threads in small for t in threads)
+    large = [(*v, 8, (1 << 22) + 4) for v in VARIANTS]
+    for (method, opt, state_sync, *_), (_, _, *threads) in zip(large, rules(large)):
+        assert threads[2] == (64 if opt == "adamw" and state_sync else 256)
