@@ -3,20 +3,22 @@
 //
 // What bounds the column kernels there: one thread walks all W rows of its
 // columns, a chunk at a time, so a launch takes about W / 2 dependent trips to
-// memory however few columns there are, and N / 1024 blocks cannot fill 152
-// SMs (W = 64, N = 60,000: 59 blocks, 32.8 us for 78 MB). Here a block owns the
-// columns of 32 loads (64 at even N, 32 at odd) and its 4 to 16 warps take
-// every R-th row, so a column's rows are loaded by R warps at once and N / 64
-// (N / 32) blocks run. The values to be averaged pass through shared memory,
-// where one thread per column adds them in worker order: the sums are those of
-// the other kernels bit for bit (partial sums per warp measured the same
-// within 10 %, but in another order). Sync step, us, column kernels -> this one,
-// CPDP SGD f32: W = 64, N = 60,000 32.8 -> 14.9 (5.2 TB/s; the bytes take 11.4
-// at the copy rate); W = 16, N = 20,000 5.54 -> 2.26; W = 200, N = 20,000 90.6 ->
-// 22.2; AdamW bf16 W = 64, N = 20,000 47 -> 10.4. What bounds it now is the trips
-// that are left, two to six per 64 rows, and the barriers between them.
+// memory however few columns there are, on N / 256 blocks of 2 warps (W = 64,
+// N = 60,000: 235). Here a block owns the columns of 32 loads (64 at even N, 32
+// at odd) and its 4 to 16 warps take every R-th row, so a column's rows are
+// loaded by R warps at once and N / 64 (N / 32) blocks run. The values to be
+// averaged pass through shared memory, where one thread per column adds them
+// in worker order: the sums are those of the other kernels bit for bit (partial
+// sums per warp measured the same within 10 %, but in another order). Sync step,
+// us, column kernel -> this one, CPDP SGD f32, state from DRAM: W = 64,
+// N = 60,000 30.6 -> 15.6 (5.0 TB/s; the bytes take 11.4 at the copy rate);
+// W = 16, N = 23,000 8.3 -> 3.5; W = 200, N = 23,000 86.5 -> 23.9; AdamW bf16
+// W = 64, N = 24,000 45 -> 11. State in L2: W = 64, N = 61,000 17.6 -> 11.1; W = 16,
+// N = 23,000 4.4 -> 2.5. What bounds it now is the trips that are left, two to
+// six per 64 rows, and the barriers between them.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -29,33 +31,43 @@ constexpr int kSplitMaxWarps = 16;
 
 // Where it is used. From 9 workers: up to 8 the column kernels need at most
 // four trips. Above these sizes the column kernels have blocks enough, and
-// their longer row segments win (ratio of sync-step times, column kernel over
-// this one): even N, W = 9: N = 60,000 1.17-1.40 for SGD, 100,000 0.85-1.18;
-// W = 16: 100,000 1.04-1.61, 200,000 0.85-1.24; W = 64: 100,000 1.26-1.72,
-// 200,000 1.04-1.27, 400,000 0.92-1.02. Odd N: W = 9 20,001 1.24-1.32, 60,001
-// 0.79-0.85; W = 24 and more 64,003 1.00-2.0.
+// their longer row segments win. Time of the column kernel (64-thread blocks)
+// over this one's, state in L2 or not, geometric mean over the variants (and
+// the worst). Even N without state reconciliation: W = 9 N = 64,000 1.4 (1.1);
+// W = 12 85,000 1.15 (0.9), 110,000 1.05 (0.8); W = 16 to 24 110,000 1.1-1.3,
+// 140,000 1.05-1.2, of them SGD with bf16 gradients (CPDP, DDP) 0.86-0.96 from
+// 82,000; W = 32 and more 140,000 1.15-1.3, 180,000 1.1-1.2, 300,000 1.0-1.15
+// (0.85). With it: W = 16 to 24 SGD 85,000 0.94-1.1 (CPDP 0.77-0.96; LocalSGD
+// bf16 1.0 and more), 140,000 0.93-1.03; AdamW 110,000 1.1-1.2 (CPDP bf16
+// 0.84-0.94); W = 32 and more SGD 140,000 1.1-1.2 (CPDP bf16 0.81-0.96 from
+// 100,000), AdamW 110,000 1.1-1.25 (LocalSGD 0.84-0.96), 140,000 1.0-1.1 (0.80).
 // Odd rows cost the column kernels more, as a row is more of 4-byte loads, and
 // this kernel holds 8 of them at once (split_deep), so its range is longer
-// at odd N: float32 gradients, SGD from 24 workers to 300,001 1.05-1.60 for
-// CPDP, 1.03-1.29 for LocalSGD, and for DDP from 9 workers 0.96-2.0; AdamW from
-// 24 workers to 420,001 1.01-1.55 for DDP and LocalSGD, for CPDP to 100,001
-// 1.03-1.22 (0.86-1.08 to 300,001) and from 100 workers to 300,001 1.0-1.26;
-// bf16 from 48 workers to 100,001 1.03-1.19 (0.89-1.05 at 150,001). State
-// reconciliation from 100 workers to 300,001, AdamW and LocalSGD: 1.02-1.45;
-// CPDP SGD 0.90-1.14, so it keeps 64,000.
-// Its offsets are 32-bit: W rows of N / V loads stay below 2^31.
+// at odd N: float32 gradients, SGD from 24 workers to 300,001 1.0-1.4 for
+// CPDP and LocalSGD, DDP from 9 workers 1.0-2.0 to 160,001, below 24 workers
+// 0.84-0.93 above; AdamW from 24 workers to 420,001 1.0-1.5 for DDP and
+// LocalSGD, for CPDP to 110,001 1.0-1.2 and from 100 workers to 300,001
+// 1.0-1.3; bf16 from 48 workers to 110,001 1.0-1.2. State reconciliation from
+// 100 workers to 300,001, AdamW and LocalSGD: 1.0-1.4; CPDP SGD 0.9-1.1, so it
+// keeps 64,000. Its offsets are 32-bit: W rows of N / V loads stay below 2^31.
 inline bool split_takes(const ReconcileCall& c) {
     const int64_t units = (c.N & 1) == 0 ? c.N >> 1 : c.N;
     if (c.W < 9 || c.W * units >= int64_t(1) << 31) return false;
-    if ((c.N & 1) == 0) return c.N <= (c.W < 16 ? 64'000 : 160'000);
-    const bool sgd = c.opt == kOptSGD, cpdp_method = c.method == kMethodCPDP;
-    int64_t limit = c.W < 24 ? 24'000 : 64'000;
+    const bool sgd = c.opt == kOptSGD, cpdp_method = c.method == kMethodCPDP, local = c.method == kMethodLocalSGD;
+    int64_t limit;
+    if ((c.N & 1) == 0) {
+        limit = c.W < 16 ? 64'000 : 160'000;
+        if (c.state_sync && (!sgd || (cpdp_method && c.bf16))) limit = std::min<int64_t>(limit, 100'000);
+        if (c.W < 32 && !local && (c.state_sync || (sgd && c.bf16))) limit = std::min<int64_t>(limit, 80'000);
+        return c.N <= limit;
+    }
+    limit = c.W < 24 ? 24'000 : 64'000;
     if (c.state_sync) {
         if (c.W >= 100 && (!sgd || !cpdp_method)) limit = 300'000;
     } else if (c.bf16) {
         if (c.W >= 48) limit = 110'000;
     } else if (sgd && (c.method == kMethodDDP || c.W >= 24)) {
-        limit = 300'000;
+        limit = c.W < 24 ? 160'000 : 300'000;
     } else if (!sgd && c.W >= 24 && !cpdp_method) {
         limit = 420'000;
     } else if (!sgd && c.W >= 100) {
@@ -67,10 +79,9 @@ inline bool split_takes(const ReconcileCall& c) {
 }
 
 // Warps per block over `tiles` blocks: more while the launch stays within
-// about one resident wave (152 SMs x 28 warps) and a warp keeps 3 rows or more
-// (CPDP SGD f32 with partial sums, us at 4 / 8 / 16 warps: W = 16, N = 32,000
-// 2.47 / 3.29 / -; W = 64, N = 32,000 10.9 / 9.5 / -; W = 200, N = 8,000 21.4 /
-// 13.7 / 11.4).
+// about one resident wave (152 SMs x 27 warps) and a warp keeps 3 rows or more
+// (CPDP SGD f32, state in L2, us at 4 / 8 / 16 warps: W = 16, N = 32,000 2.57 / 2.91 /
+// 4.65; W = 64, N = 32,000 6.15 / 5.66 / 6.84; W = 200, N = 8,000 13.3 / 9.8 / 8.5).
 inline int split_warps(int W, int64_t tiles) {
     int warps = 4;
     while (warps < kSplitMaxWarps && tiles * warps * 2 <= 4096 && W >= 3 * warps * 2) warps *= 2;

@@ -4,11 +4,10 @@ import subprocess
 
 import pytest
 
+from launch_rules import VARIANTS, edges, split_limit
 from paper_2607_21224_gb300 import build
 
 CODES = {"cpdp": 0, "localsgd": 1, "ddp": 2}
-VARIANTS = [(m, o, s, b) for m in CODES for o in ("sgd", "adamw") for s in (False, True) for b in (False, True)
-            if not (m == "ddp" and s)]
 
 PROGRAM = r"""
 #include "cpdp_shapes.cuh"
@@ -54,6 +53,15 @@ def test_no_split_call_passes_32_bit_offsets(rules):
     for (*v, W, N), got in zip(calls, taken):
         if got:
             assert W * (N // (2 if N % 2 == 0 else 1)) < 1 << 31, (*v, W, N)
+
+
+@pytest.mark.parametrize("W", [8, 9, 15, 16, 23, 24, 31, 32, 47, 48, 99, 100, 4096])
+def test_split_limits(rules, W):
+    """Both sides of every limit, for every variant."""
+    cases = [(v, odd, N, N <= split_limit(*v, W, odd))
+             for v in VARIANTS for odd in (False, True) for N in edges(split_limit(*v, W, odd), odd) if N > 0]
+    for (v, odd, N, want), (taken, *_) in zip(cases, rules([(*v, W, N) for v, _, N, _ in cases])):
+        assert taken == want, (v, W, N)
 
 
 def test_walks_alternate_only_past_what_l2_keeps(rules):

@@ -11,15 +11,16 @@ from pathlib import Path
 import pytest
 import torch
 
+from launch_rules import split_limit
 from test_ragged_reconcile_gpu import VARIANTS, _arrays, _state
 
 pytestmark = pytest.mark.gpu
 
 ROOT = Path(__file__).resolve().parents[1]
-WIDE = 160_004  # even, and past the sizes the rule takes at even N: the column kernels
+WIDE, WIDEST = 160_004, 420_004  # even, and past the sizes the rule takes: the column kernels
 
 
-def _match(W, N, wide, want):
+def _match(W, N, wide=WIDE):
     gen = torch.Generator(device="cuda").manual_seed(N * 512 + W)
     theta0 = torch.randn(wide, device="cuda", generator=gen) * 0.05
     grads = [torch.randn((W, wide), device="cuda", generator=gen) * 1e-2 for _ in range(2)]
@@ -31,8 +32,10 @@ def _match(W, N, wide, want):
                 for step in ("local_step", "reconcile"):
                     getattr(a, step)(g[:, :N].to(dtype).contiguous())
                     getattr(b, step)(g.to(dtype))
-            assert a.reconcile_kernel() in ((want,) if want else ("reconcile_split_kernel", "reconcile_scalar_kernel"))
-            assert b.reconcile_kernel() in ("reconcile_vec4_kernel", "reconcile_onepass_kernel")
+            columns = "reconcile_scalar_kernel" if N % 4 else "reconcile_vec4_kernel"
+            split = N <= split_limit(method, opt, state_sync, dtype == torch.bfloat16, W, N % 2 == 1)
+            assert a.reconcile_kernel() == ("reconcile_split_kernel" if split else columns)
+            assert b.reconcile_kernel() == "reconcile_vec4_kernel"
             for x, y in zip(_arrays(a), _arrays(b)):
                 assert torch.equal(x, y[..., :N]), (method, opt, state_sync, dtype)
 
@@ -40,31 +43,35 @@ def _match(W, N, wide, want):
 @pytest.mark.parametrize("W", [9, 15, 24, 33, 64, 65, 131])
 @pytest.mark.parametrize("N", [1, 2, 31, 33, 63, 66, 129, 4098, 23_999])
 def test_split_rows_match_the_column_kernels(N, W):
-    _match(W, N, WIDE, "reconcile_split_kernel")
+    _match(W, N)
 
 
-@pytest.mark.parametrize("W,N,want", [
-    (8, 1200, "reconcile_vec4_kernel"), (9, 64_000, "reconcile_split_kernel"), (9, 64_004, "reconcile_vec4_kernel"),
-    (16, 160_000, "reconcile_split_kernel"), (23, 24_001, None), (24, 63_999, "reconcile_split_kernel"),
-    (24, 64_001, None), (9, 159_999, None), (100, 110_001, None), (24, 109_999, None), (24, 31_999, "reconcile_split_kernel"), (24, 32_001, "reconcile_split_kernel"),
-    (24, 64_002, "reconcile_split_kernel"), (63, 8_194, "reconcile_split_kernel"), (65, 8_195, "reconcile_split_kernel"),
-    (100, 60_001, "reconcile_split_kernel"), (4096, 66, "reconcile_split_kernel")])
-def test_the_rule_that_selects_it(W, N, want):
-    if W * WIDE > 1 << 26:  # 4,096 workers: a wider problem of its own size
-        gen = torch.Generator(device="cuda").manual_seed(1)
-        with _state(W, N, "cpdp", "sgd", False) as a, _state(W // 16, N, "cpdp", "sgd", False) as b:
-            theta0 = torch.randn(N, device="cuda", generator=gen) * 0.05
-            g = torch.randn((W // 16, N), device="cuda", generator=gen) * 1e-2
-            for st, grads in ((a, g.repeat(16, 1)), (b, g)):
-                st.init_params(theta0)
-                st.local_step(grads)
-                st.reconcile(grads)
-            assert a.reconcile_kernel() == want
-            # 16 copies of 256 workers have the same means, to the rounding of 4,096-term sums
-            assert torch.allclose(a.anchor, b.anchor, rtol=0, atol=4096 * 2.0 ** -24 * float(a.anchor.abs().max()))
-            assert torch.equal(a.params, a.params[:1].expand_as(a.params))
-    else:
-        _match(W, N, WIDE, want)
+@pytest.mark.parametrize("W,N,wide", [
+    (8, 1200, WIDE), (9, 64_000, WIDE), (9, 64_004, WIDE), (16, 80_000, WIDE), (16, 80_002, WIDE), (31, 100_000, WIDE),
+    (31, 100_002, WIDE), (32, 100_004, WIDE), (16, 160_000, WIDE), (32, 160_002, WIDE), (24, 64_002, WIDE),
+    (23, 24_001, WIDE), (24, 31_999, WIDE), (24, 32_001, WIDE), (24, 63_999, WIDE), (24, 64_001, WIDE), (16, 110_001, WIDE),
+    (24, 109_999, WIDE), (48, 110_001, WIDE), (9, 159_999, WIDE), (9, 160_001, WIDE), (24, 299_999, WIDEST),
+    (24, 300_001, WIDEST), (24, 419_999, WIDEST), (24, 420_001, WIDEST), (100, 60_001, WIDE), (100, 110_001, WIDE),
+    (100, 299_999, WIDEST), (100, 300_001, WIDEST), (63, 8_194, WIDE), (65, 8_195, WIDE)])
+def test_the_rule_that_selects_it(W, N, wide):
+    """Each variant on the side of its limit where it belongs, and the same bits on both."""
+    _match(W, N, wide)
+
+
+def test_the_most_workers():
+    W, N = 4096, 66  # a wider problem would be too large: fewer workers instead
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    with _state(W, N, "cpdp", "sgd", False) as a, _state(W // 16, N, "cpdp", "sgd", False) as b:
+        theta0 = torch.randn(N, device="cuda", generator=gen) * 0.05
+        g = torch.randn((W // 16, N), device="cuda", generator=gen) * 1e-2
+        for st, grads in ((a, g.repeat(16, 1)), (b, g)):
+            st.init_params(theta0)
+            st.local_step(grads)
+            st.reconcile(grads)
+        assert a.reconcile_kernel() == "reconcile_split_kernel"
+        # 16 copies of 256 workers have the same means, to the rounding of 4,096-term sums
+        assert torch.allclose(a.anchor, b.anchor, rtol=0, atol=4096 * 2.0 ** -24 * float(a.anchor.abs().max()))
+        assert torch.equal(a.params, a.params[:1].expand_as(a.params))
 
 
 CHECKED = """
@@ -74,7 +81,7 @@ import torch
 from test_ragged_reconcile_gpu import VARIANTS, _state
 from paper_2607_21224_gb300 import cpdp
 bad = 0
-for W, N in ((9, 66), (24, 129), (65, 1001), (131, 33), (3, 1_500_006), (9, 500_003), (8, 3 * 1024 + 126)):
+for W, N in ((9, 66), (24, 129), (65, 1001), (131, 33), (24, 300_001), (32, 160_000), (3, 1_500_006), (9, 500_003), (8, 3 * 1024 + 126)):
     for method, opt, state_sync, dtype in VARIANTS:
         with _state(W, N, method, opt, state_sync) as st:
             st.init_params(torch.zeros(N, device="cuda"))
