@@ -319,9 +319,10 @@ class Worst(dict):
 
 def run_and_check(wl: wls.Workload, cols=None, tol: float = TOL, seed: int = 42,
                   steps: int | None = None, method: str = "cpdp", state_sync: bool = False,
-                  staging: int = 0, shuffle: bool = False, plain: bool = False) -> Worst:
+                  staging: int = 0, shuffle: bool = False, plain: bool = False, kernel: str | None = None) -> Worst:
     """Run an epoch (or `steps` steps) of `method` on both sides, checking every
-    step. With `plain`, the metric with no floor must meet `tol` too."""
+    step. With `plain`, the metric with no floor must meet `tol` too; with
+    `kernel`, every reconcile must have launched that one."""
     pair = Pair(wl, cols, seed, method=method, state_sync=state_sync, staging=staging, shuffle=shuffle)
     worst = Worst()
     try:
@@ -337,6 +338,8 @@ def run_and_check(wl: wls.Workload, cols=None, tol: float = TOL, seed: int = 42,
                 assert st.err <= tol, f"{wl.name} t={t}: {k} error {st.err:.3e} > {tol:.0e} ({stats})"
                 if plain:
                     assert st.plain <= tol, f"{wl.name} t={t}: {k} error without floor {st.plain:.3e} > {tol:.0e}"
+            if synced and kernel is not None:
+                assert pair.gpu.reconcile_kernel() == kernel, (wl.name, t, pair.gpu.reconcile_kernel())
             if synced:
                 assert pair.replicas_identical(), f"{wl.name} t={t}: replicas differ after reconcile"
     finally:

@@ -68,11 +68,15 @@ def test_ragged_sizes(N, W):
     run_and_check(flat(f"ragged_{N}_{W}", N, W, K=2, T=5))
 
 
-@pytest.mark.parametrize("W", [2, 5, 8, 9, 16, 32])
-def test_multi_tile_vector_path(W):
+@pytest.mark.parametrize("W,tiles,kernel", [
+    (2, 37, "reconcile_onepass_kernel"), (5, 37, "reconcile_vec4_kernel"), (8, 37, "reconcile_vec4_kernel"),
+    (9, 37, "reconcile_split_kernel"), (16, 37, "reconcile_split_kernel"), (32, 37, "reconcile_split_kernel"),
+    (9, 73, "reconcile_vec4_kernel"), (16, 197, "reconcile_vec4_kernel"), (32, 197, "reconcile_vec4_kernel")])
+def test_multi_tile_vector_path(W, tiles, kernel):
     """Vector path over many blocks with a partial last block (N/4 not a
-    multiple of the block size), W not a multiple of the 8-row chunk for 5 and 9."""
-    run_and_check(flat(f"tiles_W{W}", 4 * (256 * 37 + 11), W, K=3, T=7, tensors=5))
+    multiple of the block size), W not a multiple of the 4-row chunk for 5 and
+    9. From 9 workers the vector kernel runs past the split kernel's sizes."""
+    run_and_check(flat(f"tiles_W{W}", 4 * (256 * tiles + 11), W, K=3, T=7, tensors=5), kernel=kernel)
 
 
 def test_bf16_gradients_small():
@@ -470,14 +474,15 @@ def test_many_workers_gradient_chunks(W, method, opt, gd):
     AdamW with gradient-row chunks of 8 (bf16) or 4 (float32) held as raw
     words and 4- or 3-row state chunks, the first loaded with the gradients:
     full and partial chunks of both kinds, over several blocks with a partial
-    last one, against the oracle."""
-    N = 4 * (256 * 5 + 3)
+    last one, against the oracle. From 9 workers N lies past the sizes that the
+    split kernel takes."""
+    N = 4 * (256 * (5 if W < 9 else 73 if W < 16 else 197) + 3)
     if opt == "adamw":
         wl = flat(f"gc_{W}", N, W, K=2, T=5, grad_dtype=gd, tensors=2, lr=5e-4, weight_decay=0.05, momentum=0.0,
                   optimizer="adamw")
     else:
         wl = flat(f"gc_{W}", N, W, K=2, T=5, grad_dtype=gd, tensors=2)
-    run_and_check(wl, method=method)
+    run_and_check(wl, method=method, kernel="reconcile_vec4_kernel")
 
 
 @pytest.mark.parametrize("method", ["localsgd", "ddp"])
@@ -669,9 +674,21 @@ def test_host_gradient_pipeline_matches_device_resident():
 
 @pytest.mark.parametrize("W", [64, 257, 1024, 4096])
 def test_many_workers(W):
-    """Worker counts up to the ABI's limit (4096), vector and scalar paths."""
+    """Worker counts up to the ABI's limit (4096), pairs of columns and single
+    ones of the kernel that splits the rows across warps."""
     for N in (4 * 33, 37):
-        run_and_check(flat(f"many_{W}_{N}", N, W, K=2, T=3))
+        run_and_check(flat(f"many_{W}_{N}", N, W, K=2, T=3), kernel="reconcile_split_kernel")
+
+
+@pytest.mark.parametrize("W,N,kernel", [(64, 4 * (256 * 197 + 3), "reconcile_vec4_kernel"),
+                                        (257, 4 * (256 * 197 + 3), "reconcile_vec4_kernel"),
+                                        (64, 420_003, "reconcile_scalar_kernel"),
+                                        (257, 201_742, "reconcile_scalar_kernel")])
+def test_many_workers_column_kernels(W, N, kernel):
+    """Many workers past the split kernel's sizes: vector and ragged columns,
+    sampled against the oracle."""
+    wl = flat(f"many_{W}_{N}", N, W, K=2, T=3)
+    run_and_check(wl, cols=windows(wl, width=256, n_random=512, boundaries=0), kernel=kernel)
 
 
 def test_two_contexts_on_two_host_threads():
