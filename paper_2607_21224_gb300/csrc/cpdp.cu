@@ -237,8 +237,10 @@ cpdp_status check_grads(cpdp_ctx* ctx, const void* grads, cpdp_dtype dtype) {
 
 // The walk direction of the launch being made: where launches alternate, the
 // next one goes the other way.
-int turn(cpdp_ctx* c) {
-    return cpdp::walks_alternate(c->W, c->N, c->optimizer == CPDP_OPT_ADAMW) ? c->backwards ^= 1 : 0;
+int turn(cpdp_ctx* c, int grad_bytes) {
+    const bool alternate = cpdp::walks_alternate(c->W, c->N, c->optimizer == CPDP_OPT_ADAMW,
+                                                 c->method == CPDP_METHOD_CPDP, grad_bytes);
+    return alternate ? c->backwards ^= 1 : 0;
 }
 
 template <typename G>
@@ -251,12 +253,12 @@ cudaError_t launch_local(cpdp_ctx* c, const void* grads, cudaStream_t s, const c
         return launch(c,
                       cpdp::local_step_kernel<cpdp::kOptAdamW, G, cpdp::kLocalUnroll,
                                               cpdp::LocalWarpRuns<cpdp::kOptAdamW, G>::value, false>,
-                      grid, s, c->params, c->mom, c->exp_avg_sq, g, total, a, turn(c));
+                      grid, s, c->params, c->mom, c->exp_avg_sq, g, total, a, turn(c, sizeof(G)));
     constexpr bool warp_runs = cpdp::LocalWarpRuns<cpdp::kOptSGD, G>::value;
     auto* kernel = total >= cpdp::kOnceMinElements && total <= cpdp::kOnceMaxElements
                        ? cpdp::local_step_kernel<cpdp::kOptSGD, G, cpdp::kLocalUnroll, warp_runs, true>
                        : cpdp::local_step_kernel<cpdp::kOptSGD, G, cpdp::kLocalUnroll, warp_runs, false>;
-    return launch(c, kernel, grid, s, c->params, c->mom, static_cast<float*>(nullptr), g, total, a, turn(c));
+    return launch(c, kernel, grid, s, c->params, c->mom, static_cast<float*>(nullptr), g, total, a, turn(c, sizeof(G)));
 }
 
 // The one-pass reconcile for at most Shape::wmax workers.
@@ -267,7 +269,7 @@ cudaError_t launch_onepass(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, c
     const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N, 4);
     return cpdp::launch_shaped(
         c->pdl, cpdp::reconcile_onepass_kernel<METHOD, OPT, SS, G, Shape::wmax, Shape::min_blocks>,
-        cpdp::grid_for(nq, threads), threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
+        cpdp::grid_for(nq, threads), threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c, sizeof(G)));
 }
 
 // The vectorised reconcile in launch shape Shape, with 32-bit offsets where
@@ -286,12 +288,12 @@ cudaError_t launch_vec4(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, cons
                 cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks, Shape::late, int32_t,
                                             grad_rows, overlap>,
                 grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, static_cast<int32_t>(nq), a,
-                turn(c));
+                turn(c, sizeof(G)));
     }
     return cpdp::launch_shaped(c->pdl,
                                cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks,
                                                            Shape::late, int64_t, grad_rows, overlap>,
-                               grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c));
+                               grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c, sizeof(G)));
 }
 
 template <int METHOD, int OPT, bool SS, typename G>
@@ -341,7 +343,7 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
         return launch_vec4<cpdp::ReconcileShape<OPT, G, SS>, METHOD, OPT, SS, G>(c, g, sq, s, a, nq);
     }
     c->reconcile_kernel = "reconcile_scalar_kernel";
-    call.backwards = turn(c);
+    call.backwards = turn(c, sizeof(G));
     return cpdp::launch_reconcile_ragged(call);
 }
 

@@ -34,17 +34,19 @@ struct LocalWarpRuns {
 constexpr int64_t kOnceMinElements = 6'000'000, kOnceMaxElements = int64_t(1) << 25;
 
 // Whether a context's launches alternate their walk direction (walk_block):
-// where the replicas and optimizer states (about half of L2 and more) no longer
-// stay in L2 from one launch to the next. Below that there is nothing to gain,
-// and a run of sync steps loses, as a block's columns move to another SM, and
-// mostly to the other die, each time. Back-to-back sync steps on one state, N a
-// multiple of 4, one direction over alternating, geometric means over the
-// variants: 1 to 3 MB 0.95-0.97, 5 to 13 MB 0.97-0.98, 20 to 50 MB 0.99-1.00, 56 MB
-// 0.97, 64 MB 1.02, 70 MB 1.05, 80 MB 1.07, 87 to 110 MB 1.12-1.21, 170 MB 1.12.
-// Periods of 2 and 4 steps: 0.996-1.01 to 49 MB, 61 MB 1.014, 75 MB 1.07, 93 MB 1.13.
-constexpr int64_t kAlternateMinStateBytes = 60'000'000;
-inline bool walks_alternate(int64_t W, int64_t N, bool adamw) {
-    return W * N * (adamw ? 12 : 8) >= kAlternateMinStateBytes;
+// where a sync step's arrays (replicas, optimizer states, gradients; for CPDP
+// the anchor and velocity too) are more than L2 keeps from one launch to the
+// next. Below that there is nothing to gain, and a run of sync steps loses, as a
+// block's columns move to another SM, and mostly to the other die, each time.
+// N a multiple of 4, one direction over alternating, geometric means over the
+// variants and 1 to 64 workers, sync steps in a row on one state / periods of 2
+// and 4 steps: 1 to 10 MB 0.95-0.98 / 0.998-1.01, 30 to 60 MB 0.995-1.006 / 0.996-1.001,
+// 72 MB 0.986 / 0.996, 83 MB 0.994 / 1.009, 91 MB 1.036 / 1.034, 103 MB 1.07 / 1.07,
+// 118 MB 1.13 / 1.10, 149 MB 1.17 / 1.13. Counted in the state alone the two sides mix
+// (1 to 3 workers gain from 40 MB, 8 and more lose to 60).
+constexpr int64_t kAlternateMinBytes = 84'000'000;
+inline bool walks_alternate(int64_t W, int64_t N, bool adamw, bool cpdp_method, int grad_bytes) {
+    return W * N * ((adamw ? 12 : 8) + grad_bytes) + (cpdp_method ? 8 * N : 0) >= kAlternateMinBytes;
 }
 constexpr int64_t kMaxGrid = 0x7fffffff;
 

@@ -19,7 +19,8 @@ int main() {
     long long N;
     while (std::scanf("%d %d %d %d %d %lld", &method, &opt, &state_sync, &bf16, &W, &N) == 6) {
         c.method = method, c.opt = opt, c.state_sync = state_sync != 0, c.bf16 = bf16 != 0, c.W = W, c.N = N;
-        std::printf("%d %d", cpdp::split_takes(c) ? 1 : 0, cpdp::walks_alternate(W, N, opt == cpdp::kOptAdamW) ? 1 : 0);
+        std::printf("%d %d", cpdp::split_takes(c) ? 1 : 0,
+                    cpdp::walks_alternate(W, N, opt == cpdp::kOptAdamW, method == cpdp::kMethodCPDP, bf16 ? 2 : 4) ? 1 : 0);
         for (int columns : {1, 2, 4}) std::printf(" %d", cpdp::reconcile_threads(method, opt, state_sync, W, N, columns));
         std::printf("\n");
     }
@@ -65,15 +66,12 @@ def test_split_limits(rules, W):
 
 
 def test_walks_alternate_only_past_what_l2_keeps(rules):
-    """Below half of L2 the state is there anyway, and a block that moves to another SM each time loses by it."""
-    sizes = [(1, 7_499_999, 4_999_999), (4, 1_874_999, 1_249_999), (8, 937_499, 624_999), (60, 124_999, 83_333)]
-    below = [("cpdp", o, False, False, W, n) for W, sgd, adamw in sizes for o, n in (("sgd", sgd), ("adamw", adamw))]
-    above = [(m, o, s, b, W, n + 1) for m, o, s, b, W, n in below]
-    small = [("cpdp", "sgd", False, False, 4, 3201), ("cpdp", "sgd", False, False, 2, 1 << 20)]
-    large = [("cpdp", "sgd", False, False, 8, 23_712_932), ("localsgd", "sgd", False, False, 4, 1 << 22),
-             ("ddp", "adamw", False, True, 4096, 1 << 28)]
-    assert not any(alternates for _, alternates, *_ in rules(below + small))
-    assert all(alternates for _, alternates, *_ in rules(above + large))
+    """Below 84 MB a step's arrays are in L2 anyway, and a block that moves to another SM each time loses by it."""
+    calls = [(*v, W, N) for v in VARIANTS for W in (1, 2, 3, 8, 64, 4096)
+             for N in (3201, 30_000, 140_000, 433_007, 600_000, 1 << 20, 3_000_001, 3_750_000, 6_000_000, 1 << 28)]
+    for (method, opt, _, bf16, W, N), (_, alternates, *_) in zip(calls, rules(calls)):
+        step = W * N * ((12 if opt == "adamw" else 8) + (2 if bf16 else 4)) + (8 * N if method == "cpdp" else 0)
+        assert alternates == (step >= 84e6), (method, opt, bf16, W, N, step)
 
 
 def test_blocks_last_longer_than_the_gpu_takes_to_start_them(rules):
