@@ -18,7 +18,6 @@
 // six per 64 rows, and the barriers between them.
 #pragma once
 
-#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -31,21 +30,24 @@ constexpr int kSplitMaxWarps = 16;
 
 // Where it is used. From 9 workers: up to 8 the column kernels need at most
 // four trips. Above these sizes the column kernels have blocks enough, and
-// their longer row segments win. Time of the column kernel (64-thread blocks)
-// over this one's, state in L2 or not, geometric mean over the variants (and
-// the worst). Even N without state reconciliation: W = 9 N = 64,000 1.4 (1.1);
-// W = 12 85,000 1.15 (0.9), 110,000 1.05 (0.8); W = 16 to 24 110,000 1.1-1.3,
-// 140,000 1.05-1.2, of them SGD with bf16 gradients (CPDP, DDP) 0.86-0.96 from
-// 82,000; W = 32 and more 140,000 1.15-1.3, 180,000 1.1-1.2, 300,000 1.0-1.15
-// (0.85). With it: W = 16 to 24 SGD 85,000 0.94-1.1 (CPDP 0.77-0.96; LocalSGD
-// bf16 1.0 and more), 140,000 0.93-1.03; AdamW 110,000 1.1-1.2 (CPDP bf16
-// 0.84-0.94); W = 32 and more SGD 140,000 1.1-1.2 (CPDP bf16 0.81-0.96 from
-// 100,000), AdamW 110,000 1.1-1.25 (LocalSGD 0.84-0.96), 140,000 1.0-1.1 (0.80).
+// their longer row segments win. Sync steps in a row, time of the column kernel
+// (64-thread blocks) over this one's, geometric means over worker counts with
+// the state in L2 and out of it; N a multiple of 4 / N = 2 mod 4, whose column
+// kernel has twice the threads. W = 9 to 12, N = 64,000: SGD 1.23-1.56 / 1.01-1.64, AdamW
+// 1.38-1.80 / 1.04-1.38; 85,000: SGD 0.77-1.38 / 0.78-1.50. W = 16 to 24, 110,000:
+// AdamW 1.22-1.46 / 0.93-1.24, SGD f32 1.0-1.17 / 1.03-1.15, bf16 0.91-1.25 / 0.92-1.21,
+// state-reconciling SGD 0.85-1.17 / 0.89-1.11; 140,000: 0.91-1.38 / 0.86-1.14. W = 32 and
+// more, 140,000: 0.98-1.53 / 0.82-1.32; 180,000: 0.87-1.25 / 0.91-1.44. In a period
+// of 2 or 4 steps, where the local steps leave other lines in L2, it is further
+// ahead (N a multiple of 4): W = 20, N = 91,000 to 134,000, state-reconciling CPDP SGD
+// 1.23-1.27, W = 32, N = 154,000 1.16, W = 200, N = 108,000 1.35, state-reconciling AdamW
+// W = 24 to 48, N = 103,000 to 126,000 1.4-2.0.
 // Odd rows cost the column kernels more, as a row is more of 4-byte loads, and
 // this kernel holds 8 of them at once (split_deep), so its range is longer
 // at odd N: float32 gradients, SGD from 24 workers to 300,001 1.0-1.4 for
-// CPDP and LocalSGD, DDP from 9 workers 1.0-2.0 to 160,001, below 24 workers
-// 0.84-0.93 above; AdamW from 24 workers to 420,001 1.0-1.5 for DDP and
+// CPDP and LocalSGD; DDP from 9 workers 1.0-2.0, at 9 to 23 workers to 250,001
+// (W = 12 to 20, 150,000 to 235,000 0.98-1.45, with the state in L2 0.86-1.33; 292,000
+// 0.83); AdamW from 24 workers to 420,001 1.0-1.5 for DDP and
 // LocalSGD, for CPDP to 110,001 1.0-1.2 and from 100 workers to 300,001
 // 1.0-1.3; bf16 from 48 workers to 110,001 1.0-1.2. State reconciliation from
 // 100 workers to 300,001, AdamW and LocalSGD: 1.0-1.4; CPDP SGD 0.9-1.1, so it
@@ -53,21 +55,15 @@ constexpr int kSplitMaxWarps = 16;
 inline bool split_takes(const ReconcileCall& c) {
     const int64_t units = (c.N & 1) == 0 ? c.N >> 1 : c.N;
     if (c.W < 9 || c.W * units >= int64_t(1) << 31) return false;
-    const bool sgd = c.opt == kOptSGD, cpdp_method = c.method == kMethodCPDP, local = c.method == kMethodLocalSGD;
-    int64_t limit;
-    if ((c.N & 1) == 0) {
-        limit = c.W < 16 ? 64'000 : 160'000;
-        if (c.state_sync && (!sgd || (cpdp_method && c.bf16))) limit = std::min<int64_t>(limit, 100'000);
-        if (c.W < 32 && !local && (c.state_sync || (sgd && c.bf16))) limit = std::min<int64_t>(limit, 80'000);
-        return c.N <= limit;
-    }
-    limit = c.W < 24 ? 24'000 : 64'000;
+    if ((c.N & 1) == 0) return c.N <= (c.W < 16 ? 64'000 : 160'000);
+    const bool sgd = c.opt == kOptSGD, cpdp_method = c.method == kMethodCPDP;
+    int64_t limit = c.W < 24 ? 24'000 : 64'000;
     if (c.state_sync) {
         if (c.W >= 100 && (!sgd || !cpdp_method)) limit = 300'000;
     } else if (c.bf16) {
         if (c.W >= 48) limit = 110'000;
     } else if (sgd && (c.method == kMethodDDP || c.W >= 24)) {
-        limit = c.W < 24 ? 160'000 : 300'000;
+        limit = c.W < 24 ? 250'000 : 300'000;
     } else if (!sgd && c.W >= 24 && !cpdp_method) {
         limit = 420'000;
     } else if (!sgd && c.W >= 100) {

@@ -11,13 +11,7 @@ def split_limit(method, opt, state_sync, bf16, W, odd):
     if W < 9:
         return 0
     if not odd:
-        if W < 16:
-            return 64_000
-        if W < 32 and method != "localsgd" and (state_sync or (opt == "sgd" and bf16)):
-            return 80_000
-        if state_sync and (opt == "adamw" or (method == "cpdp" and bf16)):
-            return 100_000
-        return 160_000
+        return 64_000 if W < 16 else 160_000
     if state_sync:
         return 300_000 if W >= 100 and (opt, method) != ("sgd", "cpdp") else 64_000 if W >= 24 else 24_000
     if bf16:
@@ -25,7 +19,7 @@ def split_limit(method, opt, state_sync, bf16, W, odd):
     if opt == "sgd":
         if W >= 24:
             return 300_000
-        return 160_000 if method == "ddp" else 110_000 if method == "localsgd" and W >= 16 else 24_000
+        return 250_000 if method == "ddp" else 110_000 if method == "localsgd" and W >= 16 else 24_000
     if W >= 24 and method != "cpdp":
         return 420_000
     return 300_000 if W >= 100 else 110_000 if W >= 16 else 24_000
