@@ -29,8 +29,14 @@ struct Ragged {
 
     template <int METHOD, int OPT, bool SS, typename G, int V>
     cudaError_t shaped() const {
-        if (c.W == 1) return by_size<RaggedShapeW1, RaggedShapeW1, METHOD, OPT, SS, G, V>();
-        using Narrow = RaggedShapeNarrow<V, OPT, SS, G>;
+        if (c.W == 1) {
+            if constexpr (V == 1 && SS)
+                if (c.N > ragged_narrow_columns<METHOD, V, OPT, SS>(1) && c.N <= kRaggedW1Columns)
+                    return launch_shape<RaggedShapeW1States, METHOD, OPT, SS, G, V, 1, int32_t>(c);
+            return by_size<RaggedShapeW1, RaggedShapeW1, METHOD, OPT, SS, G, V>();
+        }
+        if (c.W == 2) return by_size<RaggedShapeW2, RaggedShape<V, OPT, SS, G, false>, METHOD, OPT, SS, G, V>();
+        using Narrow = RaggedShapeNarrow<METHOD, V, OPT, SS, G>;
         using Few = RaggedShape<V, OPT, SS, G, false>;
         using Many = RaggedShape<V, OPT, SS, G, true>;
         if constexpr (Many::rows != Few::rows)
@@ -40,7 +46,7 @@ struct Ragged {
     // one load per thread and row for few columns, kRaggedColumns / 32 columns per thread for more
     template <typename Narrow, typename Wide, int METHOD, int OPT, bool SS, typename G, int V>
     cudaError_t by_size() const {
-        if (c.N <= ragged_narrow_columns<V, OPT, SS>(c.W) && static_cast<int64_t>(c.W) * c.N < (int64_t(1) << 30))
+        if (c.N <= ragged_narrow_columns<METHOD, V, OPT, SS>(c.W) && static_cast<int64_t>(c.W) * c.N < (int64_t(1) << 30))
             return launch_shape<Narrow, METHOD, OPT, SS, G, V, 1, int32_t>(c);
         constexpr int U = kRaggedColumns / (32 * V);
         // the largest offset formed is below W rows plus one grid-wide step

@@ -291,48 +291,77 @@ struct RaggedShape {
     static constexpr bool late = true;
 };
 
-// Few columns: at 4 columns per thread N = 300,000 gives an SM two of the four 256-thread
-// blocks it can hold, so up to ragged_narrow_columns a thread owns one load's
-// columns instead and 4-row chunks keep it busy (W = 8, N = 100,001, us, one
-// column and one row at a time / 4 columns / this: CPDP SGD f32 5.15 / 5.87 /
-// 4.29; N = 300,002 AdamW bf16 15.1 / 16.2 / 12.7). The lines are where the two
-// cross (SGD f32, W = 64: the wide shape takes 62.1 us at N = 200,001, where it
-// fills SMs unevenly, the narrow one 41.1 at 150,001; W = 8: N = 300,001 12.4
-// narrow, 11.6 wide; N = 300,002 10.3
-// and 11.8; N = 600,002 18.7 and 17.8; AdamW f32 at N = 600,002 25.0 and 30.9,
-// at 2,000,002 76.5 and 75.5). State-reconciling SGD stores nothing inside its
-// row loop and holds little per column, so 1-row chunks at 8 blocks of single
-// columns are as good as any up to 700,000 odd columns below 24 workers (W = 8,
-// N = 300,001 10.4 us; at 6 blocks 12.0, 4-row chunks 12.4; W = 141, N = 351,435
-// 249, the wide shape 209) and beat pairs up to
-// kRaggedSinglesColumns even ones (W = 4, N = 100,002 2.5 us against 2.8).
-// State-reconciling AdamW is short of registers for the overlapped chunk and
-// takes 5 blocks without it (W = 8, N = 300,001 15.2 and 14.0 us for float32
-// and bf16 gradients, overlapped at 4 blocks 15.9 and 14.5).
+// Few columns: at 4 columns per thread N = 300,000 leaves an SM half of the warps
+// it can hold, so up to ragged_narrow_columns a thread owns one load's columns
+// instead and 4-row chunks keep it busy (W = 8, N = 100,001, us, one column and
+// one row at a time / 4 columns / this: CPDP SGD f32 5.15 / 5.87 / 4.29;
+// N = 300,002 AdamW bf16 15.1 / 16.2 / 12.7). The lines are where the two cross
+// (geometric means over method and gradient type, time of a kernel with one
+// column and one row per thread over: this shape, 4 columns). SGD, odd N, sync
+// steps in a row: W = 3 to 6 N = 200,000 to 260,000 1.02-1.12, 1.08-1.17, 260,000 to
+// 330,000 0.95-1.09, 1.04-1.15, 330,000 to 430,000 1.07-1.26, 1.07-1.14; in periods of 2
+// and 4 steps (CPDP and LocalSGD, W = 3 to 16) this shape has 0.97-1.09 from 229,000 to
+// 249,000, 4 columns 0.77-0.96 from 259,000 to 325,000 and 1.0-1.1 above. W = 2 from
+// 260,000 0.99, 1.10. AdamW, odd N, W = 3 to 6, 260,000 to 330,000 0.95-1.07, 0.84-0.93,
+// 330,000 to 430,000 1.02-1.12, 0.90-0.98, W = 3, 410,000, periods 0.93, 0.99.
+// State-reconciling SGD stores nothing inside its row loop and holds little
+// per column, so 1-row chunks at 8 blocks of single columns are as good as any
+// up to 700,000 odd columns below 24 workers (W = 8, N = 300,001 10.4 us; at 6
+// blocks 12.0; W = 141, N = 351,435 249, the wide shape 209) and beat pairs up to
+// kRaggedSinglesColumns even ones. LocalSGD with bf16 gradients loads a
+// gradient row with each state row and wants 4 of them in flight (against one
+// column and one row per thread, to 60,000, 150,000, 205,000, 560,000 columns,
+// W = 6 to 14: 1-row chunks 0.90 0.94 0.93 1.00, 4-row chunks at 5 blocks 1.06 0.96
+// 1.23 1.00). State-reconciling AdamW is short of registers for the overlapped
+// chunk and takes 5 blocks without it (W = 8, N = 300,001 15.2 and 14.0 us for
+// float32 and bf16 gradients, overlapped at 4 blocks 15.9 and 14.5).
 constexpr int64_t kRaggedSinglesColumns = 200'000;
-template <int V, int OPT, bool SS>
+template <int METHOD, int V, int OPT, bool SS>
 inline int64_t ragged_narrow_columns(int W) {
     if (W == 1) return V == 2 ? 450'000 : 150'000;
     if (V == 2) return OPT == kOptAdamW || SS ? 1'500'000 : 500'000;
+    if (W == 2) return OPT == kOptAdamW ? 450'000 : 260'000;
     if (OPT == kOptAdamW) return 400'000;
-    return SS && W < 24 ? 700'000 : 250'000;
+    return SS && W < 24 ? 700'000 : METHOD == kMethodDDP ? 250'000 : 330'000;
 }
-template <int V, int OPT, bool SS, typename G>
+template <int METHOD, int V, int OPT, bool SS, typename G>
 struct RaggedShapeNarrow {
-    static constexpr bool one_row = SS && OPT == kOptSGD, plain_chunks = V == 1 && SS && OPT == kOptAdamW;
+    static constexpr bool f32 = std::is_same<G, float>::value;
+    static constexpr bool row_loads = METHOD == kMethodLocalSGD && SS && OPT == kOptSGD && !f32;
+    static constexpr bool one_row = SS && OPT == kOptSGD && !row_loads;
+    static constexpr bool plain_chunks = row_loads || (V == 1 && SS && OPT == kOptAdamW);
     static constexpr bool overlap = !one_row && !plain_chunks;
     static constexpr int rows = one_row ? 1 : 4;
     static constexpr int min_blocks = plain_chunks ? 5 : V == 1 && one_row ? 8 : 4;
-    static constexpr int grad_rows = one_row ? 1 : std::is_same<G, float>::value ? 4 : 8;
+    static constexpr int grad_rows = one_row || row_loads ? rows : f32 ? 4 : 8;
     static constexpr bool late = true;
+};
+
+// Two workers, few columns: both rows of everything in one trip. Time of a
+// kernel with one column and one row per thread over: the narrow shape above,
+// this one. N = 40,000, 130,000, 180,000, 230,000, odd: state-reconciling SGD 0.93 0.96
+// 1.03 1.02, 1.02 0.91 1.15 1.13; SGD 1.13 1.12 0.93 0.87, 1.16 1.12 1.21 1.21; AdamW
+// 1.04 1.06 0.93 0.90, 1.00 1.05 1.22 1.18; state-reconciling AdamW 1.00 0.90 1.17
+// 0.89, 1.01 0.93 1.19 1.18. N = 2 mod 4, to 1.05 M: 0.91-1.22, 0.92-1.43.
+struct RaggedShapeW2 {
+    static constexpr int rows = 2, min_blocks = 6, grad_rows = 2;
+    static constexpr bool late = true, overlap = true;
 };
 
 // One worker: all rows of a column in one round trip (N = 23.7 M, SGD f32
 // 4,244 -> 6,681 GB/s at odd N, 4,251 -> 6,656 at N = 2 mod 4; AdamW bf16
-// 4,579 -> 6,609 and 4,582 -> 6,616).
+// 4,579 -> 6,609 and 4,582 -> 6,616). State reconciliation at odd N keeps one
+// column per thread without it between 150,000 and kRaggedW1Columns (one column
+// and one row per thread over 4 columns / this: AdamW N = 180,000 0.81 / 0.97,
+// 290,000 0.91 / 0.98; SGD 180,000 0.95 / 1.06, 240,000 0.92 / 1.04).
 struct RaggedShapeW1 {
     static constexpr int rows = 1, min_blocks = 4, grad_rows = 1;
     static constexpr bool late = false, overlap = true;
+};
+constexpr int64_t kRaggedW1Columns = 330'000;
+struct RaggedShapeW1States {
+    static constexpr int rows = 1, min_blocks = 8, grad_rows = 1;
+    static constexpr bool late = true, overlap = false;
 };
 
 // One round trip for few workers (reconcile_onepass_kernel: every row of a

@@ -13,6 +13,7 @@ PROGRAM = r"""
 #include "cpdp_shapes.cuh"
 #include "cpdp_split.cuh"
 #include <cstdio>
+#include <type_traits>
 int main() {
     cpdp::ReconcileCall c{};
     int method, opt, state_sync, bf16, W;
@@ -22,7 +23,21 @@ int main() {
         std::printf("%d %d", cpdp::split_takes(c) ? 1 : 0,
                     cpdp::walks_alternate(W, N, opt == cpdp::kOptAdamW, method == cpdp::kMethodCPDP, bf16 ? 2 : 4) ? 1 : 0);
         for (int columns : {1, 2, 4}) std::printf(" %d", cpdp::reconcile_threads(method, opt, state_sync, W, N, columns));
-        std::printf("\n");
+        const auto narrow = [&](auto adamw, auto states) {
+            constexpr int O = decltype(adamw)::value ? cpdp::kOptAdamW : cpdp::kOptSGD;
+            constexpr bool S = decltype(states)::value;
+            const bool ddp = method == cpdp::kMethodDDP;
+            std::printf(" %lld %lld\n",
+                        (long long)(ddp ? cpdp::ragged_narrow_columns<cpdp::kMethodDDP, 1, O, S>(W)
+                                        : cpdp::ragged_narrow_columns<cpdp::kMethodCPDP, 1, O, S>(W)),
+                        (long long)cpdp::ragged_narrow_columns<cpdp::kMethodCPDP, 2, O, S>(W));
+        };
+        const std::true_type yes;
+        const std::false_type no;
+        if (opt)
+            state_sync ? narrow(yes, yes) : narrow(yes, no);
+        else
+            state_sync ? narrow(no, yes) : narrow(no, no);
     }
 }
 """
@@ -31,7 +46,8 @@ int main() {
 @pytest.fixture(scope="module")
 def rules(tmp_path_factory):
     """rules(calls) for each call (method, opt, state_sync, bf16, W, N): taken by the split kernel; walk direction
-    alternates; threads per block at 1, 2 and 4 columns per thread."""
+    alternates; threads per block at 1, 2 and 4 columns per thread; columns to which a ragged row gets one load per
+    thread, odd N and N = 2 mod 4."""
     folder = tmp_path_factory.mktemp("launch_rules")
     source, program = folder / "rules.cu", folder / "rules"
     source.write_text(PROGRAM)
@@ -79,12 +95,22 @@ def test_blocks_last_longer_than_the_gpu_takes_to_start_them(rules):
     columns 256 threads, except where smaller blocks gain."""
     sizes = [65_537, 100_000, 855_424, 1 << 20, 1_800_000, 1 << 22]
     calls = [(*v, W, N) for v in VARIANTS for W in (1, 2, 3, 4, 5, 6, 8, 64) for N in sizes]
-    for (*v, W, N), (_, _, *threads) in zip(calls, rules(calls)):
+    for (*v, W, N), (_, _, *threads, _, _) in zip(calls, rules(calls)):
         for columns, t in zip((1, 2, 4), threads):
             assert t in (64, 128, 256) and (t == 256 or t * columns * W >= 768), (*v, W, N, columns, t)
             assert t == 64 or t // 2 * columns * W < 768, (*v, W, N, columns, t)
     small = rules([(*v, W, N) for v in VARIANTS for W in (1, 2, 64) for N in (1, 3201, 65_536)])
-    assert all(t == 64 for _, _, *threads in small for t in threads)
+    assert all(t == 64 for _, _, *threads, _, _ in small for t in threads)
     large = [(*v, 8, (1 << 22) + 4) for v in VARIANTS]
-    for (method, opt, state_sync, *_), (_, _, *threads) in zip(large, rules(large)):
+    for (method, opt, state_sync, *_), (_, _, *threads, _, _) in zip(large, rules(large)):
         assert threads[2] == (64 if opt == "adamw" and state_sync else 256)
+
+
+@pytest.mark.parametrize("method,opt,state_sync,W,odd,even", [
+    ("cpdp", "sgd", False, 1, 150_000, 450_000), ("ddp", "sgd", False, 2, 260_000, 500_000),
+    ("cpdp", "sgd", False, 3, 330_000, 500_000), ("ddp", "sgd", False, 3, 250_000, 500_000),
+    ("localsgd", "sgd", True, 2, 260_000, 1_500_000), ("cpdp", "sgd", True, 3, 700_000, 1_500_000),
+    ("cpdp", "sgd", True, 24, 330_000, 1_500_000), ("cpdp", "adamw", False, 2, 450_000, 1_500_000),
+    ("localsgd", "adamw", True, 7, 400_000, 1_500_000), ("ddp", "adamw", False, 8, 400_000, 1_500_000)])
+def test_columns_to_which_a_ragged_row_gets_one_load_per_thread(rules, method, opt, state_sync, W, odd, even):
+    assert rules([(method, opt, state_sync, False, W, 100_001)])[0][-2:] == (odd, even)

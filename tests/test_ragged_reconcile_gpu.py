@@ -32,10 +32,13 @@ def _arrays(st):
     return [x for x in (st.params, st.mom, st.anchor, st.slow_v, getattr(st, "exp_avg_sq", None)) if x is not None]
 
 
-@pytest.mark.parametrize("W", [1, 3, 7, 8])
-@pytest.mark.parametrize("N", [2, 31, 33, 62, 66, 127, 130, 255, 1022, 1025, 3 * 1024 + 126, 200_001, 400_003, 500_002,
-                               700_002, 1_500_002])
-def test_ragged_columns_match_the_vector_kernel(N, W):
+@pytest.mark.parametrize("W,N", [(W, N) for W in (1, 3, 7, 8)
+                                 for N in (2, 31, 33, 62, 66, 127, 130, 255, 1022, 1025, 3 * 1024 + 126, 200_001, 400_003,
+                                           500_002, 700_002, 1_500_002)]
+                         + [(1, 150_003), (1, 330_001), (1, 450_002), (2, 1), (2, 126), (2, 4099), (2, 100_002), (2, 260_001),
+                            (2, 330_003), (2, 450_001), (2, 1_500_006), (3, 249_999), (4, 250_001), (7, 329_999), (8, 330_001), (8, 399_999)]
+                         + [(W, N) for W in (9, 17, 33) for N in (420_003, 500_002, 1_500_002)])
+def test_ragged_columns_match_the_vector_kernel(W, N):
     M = (N + 3) // 4 * 4  # the vector kernel's size: the same columns and up to 3 more
     gen = torch.Generator(device="cuda").manual_seed(N * 16 + W)
     theta0 = torch.randn(M, device="cuda", generator=gen) * 0.05
