@@ -298,11 +298,11 @@ cpdp_status cpdp_set_reconcile_shuffle(cpdp_ctx *ctx, int enable);
  * "reconcile_onepass_kernel", "reconcile_scalar_kernel",
  * "reconcile_split_kernel" (many workers over few columns),
  * "reconcile_tma_kernel" or "reconcile_shuffle_kernel"; "" before the first
- * one. The launch shape is chosen per worker count, method, optimizer, state
- * reconciliation and gradient type, so this tells a caller (a profile, a
- * benchmark) which kernel ran. The string is static: never freed, valid for
- * the life of the library. Host-only; an invalid ctx or a NULL name returns
- * CPDP_EINVAL and leaves *name unchanged.
+ * one. Kernel and launch shape are chosen per worker count, parameter count,
+ * method, optimizer, state reconciliation and gradient type, so this tells a
+ * caller (a profile, a benchmark) which kernel ran. The string is static:
+ * never freed, valid for the life of the library. Host-only; an invalid ctx or
+ * a NULL name returns CPDP_EINVAL and leaves *name unchanged.
  */
 cpdp_status cpdp_reconcile_kernel(const cpdp_ctx *ctx, const char **name);
 

@@ -269,7 +269,8 @@ cudaError_t launch_onepass(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, c
     const int threads = cpdp::reconcile_threads(METHOD, OPT, SS, c->W, c->N, 4);
     return cpdp::launch_shaped(
         c->pdl, cpdp::reconcile_onepass_kernel<METHOD, OPT, SS, G, Shape::wmax, Shape::min_blocks>,
-        cpdp::grid_for(nq, threads), threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c, sizeof(G)));
+        cpdp::grid_for(nq, threads), threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a,
+        turn(c, sizeof(G)));
 }
 
 // The vectorised reconcile in launch shape Shape, with 32-bit offsets where
@@ -293,7 +294,8 @@ cudaError_t launch_vec4(cpdp_ctx* c, const G* g, float* sq, cudaStream_t s, cons
     return cpdp::launch_shaped(c->pdl,
                                cpdp::reconcile_vec4_kernel<METHOD, OPT, SS, G, Shape::rows, Shape::min_blocks,
                                                            Shape::late, int64_t, grad_rows, overlap>,
-                               grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a, turn(c, sizeof(G)));
+                               grid, threads, 0, s, c->params, c->mom, sq, g, c->anchor, c->slow_v, c->W, nq, a,
+                               turn(c, sizeof(G)));
 }
 
 template <int METHOD, int OPT, bool SS, typename G>
@@ -303,7 +305,7 @@ cudaError_t launch_reconcile_variant(cpdp_ctx* c, const void* grads, cudaStream_
     const G* g = static_cast<const G*>(grads);
     // what the kernels of the other translation units take
     cpdp::ReconcileCall call{c->pdl, METHOD, OPT, SS, sizeof(G) == 2, c->W, c->N, c->params, c->mom, sq, grads,
-                                   c->anchor, c->slow_v, a, 0, s};
+                             c->anchor, c->slow_v, a, 0, s};
     if (cpdp::split_takes(call)) {
         c->reconcile_kernel = "reconcile_split_kernel";
         return cpdp::launch_reconcile_split(call);
@@ -379,7 +381,7 @@ cudaError_t launch_reconcile_tma(cpdp_ctx* c, const float* grads, cudaStream_t s
     c->tma_withheld_tile = -1;
     c->reconcile_kernel = "reconcile_tma_kernel";
     return cpdp::launch_shaped(c->pdl, cpdp::reconcile_tma_kernel, grid, cpdp::kTmaThreads, c->tma_smem, s, c->params,
-                         c->mom, grads, c->anchor, c->slow_v, c->W, c->N, c->tma_stages, withheld, a);
+                               c->mom, grads, c->anchor, c->slow_v, c->W, c->N, c->tma_stages, withheld, a);
 }
 
 cudaError_t launch_reconcile_shuffle(cpdp_ctx* c, const float* grads, cudaStream_t s, const cpdp::StepArgs& step) {
@@ -396,7 +398,7 @@ template <typename G, int CH, int MB>
 cudaError_t launch_floor_columns(float* params, float* mom, float* sq, const void* grads, float* anchor, float* slow_v,
                                  int W, int64_t nq, cudaStream_t s) {
     return cpdp::launch_shaped(true, cpdp::floor_columns_kernel<G, CH, MB>, cpdp::grid_for(nq, cpdp::kThreads),
-                         cpdp::kThreads, 0, s, params, mom, sq, static_cast<const G*>(grads), anchor, slow_v, W, nq);
+                               cpdp::kThreads, 0, s, params, mom, sq, static_cast<const G*>(grads), anchor, slow_v, W, nq);
 }
 
 template <typename G>
@@ -1025,7 +1027,7 @@ cpdp_status cpdp_floor_stream(const float* const* in, int n_in, const uint16_t* 
     const int64_t nq = n >> 2;
     const unsigned g = grid != 0 ? grid : cpdp::grid_for(nq, cpdp::kThreads);
     const cudaError_t e = cpdp::launch_shaped(true, cpdp::floor_stream_kernel, g, cpdp::kThreads, 0,
-                                        static_cast<cudaStream_t>(stream), rows, nq);
+                                              static_cast<cudaStream_t>(stream), rows, nq);
     const cudaError_t e2 = e != cudaSuccess ? e : cudaGetLastError();
     if (e2 != cudaSuccess) return set_error(nullptr, CPDP_ECUDA, "floor_stream launch: %s", cudaGetErrorString(e2));
     return CPDP_OK;
@@ -1033,7 +1035,7 @@ cpdp_status cpdp_floor_stream(const float* const* in, int n_in, const uint16_t* 
 
 cpdp_status cpdp_floor_empty(unsigned grid, void* stream) {
     const cudaError_t e = cpdp::launch_shaped(true, cpdp::floor_empty_kernel, grid != 0 ? grid : 1u, cpdp::kThreads, 0,
-                                        static_cast<cudaStream_t>(stream));
+                                              static_cast<cudaStream_t>(stream));
     const cudaError_t e2 = e != cudaSuccess ? e : cudaGetLastError();
     if (e2 != cudaSuccess) return set_error(nullptr, CPDP_ECUDA, "floor_empty launch: %s", cudaGetErrorString(e2));
     return CPDP_OK;

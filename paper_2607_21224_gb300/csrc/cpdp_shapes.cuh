@@ -24,21 +24,24 @@ struct LocalWarpRuns {
     static constexpr bool value = OPT == kOptAdamW && !std::is_same<G, float>::value;
 };
 
-// The local step's gradients leave L2 first (SGD) while the state is larger
-// than L2 keeps beside them and small enough for a part that matters to stay
-// from one step to the next. K = 4 periods, time without / with: W * N = 6 M
-// elements 1.00-1.02, 8 M 1.02-1.06, 12 M 1.02-1.04, 16 M 1.02, 24 M 1.01,
-// 33 M 1.00-1.01, 95 M (ResNet-50, 4 workers) 0.99, 190 M 0.99; 3 to 5 M
-// 0.97-1.04. AdamW gains 0.6 % at best; the reconcile, which reads fewer
-// gradients per state byte, 1 % at best.
+// The local step's gradients leave L2 first (SGD) while the state (8 bytes an
+// element with either gradient type) is larger than L2 keeps beside them and
+// small enough for a part that matters to stay from one step to the next.
+// Periods of 2 and 4 steps, 1 to 16 workers, time without / with, geometric
+// mean (and the worst), float32 and bf16 gradients: W * N = 4 M elements 1.005
+// (0.965) and 0.988 (0.966), 5.4 M 1.04 (0.97) and 1.00 (0.97), 6.6 M 1.07 (1.00)
+// and 1.016 (0.99), 8.5 M 1.07 (1.00) and 1.04 (1.00), 13 M 1.03 and 1.03, 20 M 1.014
+// and 1.010, 32 M 1.004 and 1.004, 45 M 0.998 and 0.997; 95 M (ResNet-50, 4 workers)
+// 0.99. AdamW gains 0.6 % at best; the reconcile, which reads fewer gradients per
+// state byte, 1 % at best.
 constexpr int64_t kOnceMinElements = 6'000'000, kOnceMaxElements = int64_t(1) << 25;
 
 // Whether a context's launches alternate their walk direction (walk_block):
 // where a sync step's arrays (replicas, optimizer states, gradients; for CPDP
 // the anchor and velocity too) are more than L2 keeps from one launch to the
 // next. Below that there is nothing to gain, and a run of sync steps loses, as a
-// block's columns move to another SM, and mostly to the other die, each time.
-// N a multiple of 4, one direction over alternating, geometric means over the
+// block's columns move to another SM each time (the likely cost: lines that come
+// from the other die's half of L2). N a multiple of 4, one direction over alternating, geometric means over the
 // variants and 1 to 64 workers, sync steps in a row on one state / periods of 2
 // and 4 steps: 1 to 10 MB 0.95-0.98 / 0.998-1.01, 30 to 60 MB 0.995-1.006 / 0.996-1.001,
 // 72 MB 0.986 / 0.996, 83 MB 0.994 / 1.009, 91 MB 1.036 / 1.034, 103 MB 1.07 / 1.07,
