@@ -37,17 +37,19 @@ struct LocalWarpRuns {
 constexpr int64_t kOnceMinElements = 6'000'000, kOnceMaxElements = int64_t(1) << 25;
 
 // Whether a context's launches alternate their walk direction (walk_block):
-// where a sync step's arrays (replicas, optimizer states, gradients; for CPDP
-// the anchor and velocity too) are more than L2 keeps from one launch to the
-// next. Below that there is nothing to gain, and a run of sync steps loses, as a
-// block's columns move to another SM each time (the likely cost: lines that come
-// from the other die's half of L2). N a multiple of 4, one direction over alternating, geometric means over the
-// variants and 1 to 64 workers, sync steps in a row on one state / periods of 2
-// and 4 steps: 1 to 10 MB 0.95-0.98 / 0.998-1.01, 30 to 60 MB 0.995-1.006 / 0.996-1.001,
-// 72 MB 0.986 / 0.996, 83 MB 0.994 / 1.009, 91 MB 1.036 / 1.034, 103 MB 1.07 / 1.07,
-// 118 MB 1.13 / 1.10, 149 MB 1.17 / 1.13. Counted in the state alone the two sides mix
-// (1 to 3 workers gain from 40 MB, 8 and more lose to 60).
-constexpr int64_t kAlternateMinBytes = 84'000'000;
+// not where a sync step's arrays (replicas, optimizer states, gradients; for
+// CPDP the anchor and velocity too) are few enough for L2 to keep them from one
+// launch to the next whatever else it holds. There a run of sync steps loses by
+// it, as a block's columns move to another SM each time (the likely cost: lines
+// that come from the other die's half of L2). N a multiple of 4, one direction
+// over alternating, geometric means over the variants and 1 to 64 workers, sync
+// steps in a row on one state / periods of 2 and 4 steps: 1 to 10 MB 0.95-0.98 /
+// 0.998-1.01, 24 MB 0.992 / 0.998, 30 to 60 MB 0.995-1.006 / 0.996-1.001, 72 MB 0.986 /
+// 0.996, 83 MB 0.994 / 1.009, 91 MB 1.036 / 1.034, 103 MB 1.07 / 1.07, 118 MB 1.13 / 1.10,
+// 149 MB 1.17 / 1.13. Where several states share L2 it gains from less: three of
+// 2 workers and 2^20 columns in turn (34 MB a step) take 13.77 us a period walking
+// one way and 13.61 alternating.
+constexpr int64_t kAlternateMinBytes = 30'000'000;
 inline bool walks_alternate(int64_t W, int64_t N, bool adamw, bool cpdp_method, int grad_bytes) {
     return W * N * ((adamw ? 12 : 8) + grad_bytes) + (cpdp_method ? 8 * N : 0) >= kAlternateMinBytes;
 }

@@ -1,5 +1,5 @@
 """Launches of a context alternate between walking the arrays forwards and
-backwards where a step's arrays take 84 MB and more; the direction must not
+backwards where a step's arrays take 30 MB and more; the direction must not
 change a bit. One context takes a step more than the other before both start
 over, so the same steps run in opposite directions."""
 import pytest
